@@ -23,6 +23,7 @@ struct fhd_cipher {
     int device = 0;
     uint32_t n = 32;
     double h = 0.01;
+    fhd::IntStepTab tab{};   // of h
     uint32_t u[4] = {20, 20, 40, 20};
     double key_ic[5] = {0, 0, 0, 0, 0};
     std::vector<StreamState> mirror;   // host copy of gamma (and initial state)
@@ -375,6 +376,7 @@ int init_common(const double ic[5], uint32_t n, double h, const uint32_t u[4], f
     c->partition = device_partition(dev) != nullptr;
     c->n = n;
     c->h = h;
+    c->tab = fhd::int_step_tab(h);
     for (int m = 0; m < 4; ++m) c->u[m] = u[m];
     for (int m = 0; m < 5; ++m) c->key_ic[m] = ic[m];
     e = cudaMalloc(&c->d_status, sizeof(unsigned));
@@ -508,6 +510,7 @@ int run_frames(fhd_cipher *c, uint32_t count, const fhd_frame *frames, void *str
         b.hstep = c->h;
         b.hhalf = c->h / 2.0;
         b.hsixth = c->h / 6.0;
+        b.tab = c->tab;
         for (int q = 0; q < 4; ++q) b.u[q] = c->u[q];
         uint64_t need = 0;
         for (uint32_t k = 0; k < m; ++k) {
@@ -665,6 +668,7 @@ int persistent_side(fhd_cipher *c, uint32_t count, const fhd_frame *frames, bool
     S.hstep = c->h;
     S.hhalf = c->h / 2.0;
     S.hsixth = c->h / 6.0;
+    S.tab = c->tab;
     for (int q = 0; q < 4; ++q) S.u[q] = c->u[q];
     S.states = c->d_states;
     S.status = c->d_status;
@@ -1558,6 +1562,7 @@ static int keystream_one(const double *IR, double gamma, const fhd_params *param
     b.hstep = h;
     b.hhalf = h / 2.0;
     b.hsixth = h / 6.0;
+    b.tab = fhd::int_step_tab(h);
     FrameDesc &d = b.f[0];
     d.IR = const_cast<double *>(IR);
     d.D = D;

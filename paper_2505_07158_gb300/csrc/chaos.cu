@@ -35,13 +35,22 @@
 // per stage, took ~3.5k).  In the combination, acc + 2 k is one fma(k, 2, acc):
 // 2 k is exact, so it equals the separate doubling and add whenever 2 k is
 // finite (an overflowing 2 k makes the definition's state non-finite anyway).
+//
+// LHCS_m, the trajectory kernel and the one-pair worker kernel step on the integer pipes instead (Chains in
+// chaos_dev.cuh, lorenz_int.cuh): ~1.6k cycles a step, bit-identical.  That costs issue slots, which a warp that
+// has its sub-partition to itself does not miss; the worker-pair launches that fill the GPU with chains keep the
+// binary64 steps above, six or eight chains to a warp.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
 #include "chaos_dev.cuh"
 
 namespace fhd {
 namespace {
 
 // K2a: one warp per stream of the batch; the stream's frames in call order.
-__global__ void __launch_bounds__(32) master_kernel(const __grid_constant__ Batch b, StreamState *states,
+__global__ void __launch_bounds__(32, 1) master_kernel(const __grid_constant__ Batch b, StreamState *states,
                                                     unsigned *status) {
     __shared__ __align__(16) uint8_t H[32];
     if (blockIdx.x >= b.groups) return;
@@ -49,17 +58,20 @@ __global__ void __launch_bounds__(32) master_kernel(const __grid_constant__ Batc
 }
 
 // fhd_master: one warp, one state of 5 doubles (x, y, z, w, gamma).
-__global__ void __launch_bounds__(32) master_raw_kernel(double *state5, const uint8_t *Hg, uint32_t n, Rk4 c,
-                                                        uint4 u4, double *IR, unsigned *status) {
+__global__ void __launch_bounds__(32, 1) master_raw_kernel(double *state5, const uint8_t *Hg, uint32_t n, Rk4 c,
+                                                        const __grid_constant__ IntStepTab tab, uint4 u4, double *IR,
+                                                        unsigned *status) {
     __shared__ __align__(16) uint8_t H[32];
     const int lane = threadIdx.x;
     H[lane] = Hg[lane];
     __syncwarp();
     const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
     const double gamma = state5[4];
-    const LaneRole role = lane_role(lane, gamma);
+    Chains ch;
+    ch.init(lane, lane < 4, gamma, c, tab);
+    const bool use_int = Chains::usable(lane < 4, gamma, tab);
     double s = lane_init(lane, lane < 4 ? state5[lane] : 0.0);
-    master_frame(s, lane, role, H, u, n, c, IR);
+    master_frame(s, lane, ch, use_int, H, u, n, IR);
     if (lane < 4) {
         state5[lane] = s;
         if (!finite(s) && status) atomicOr(status, kStatusNonFinite);
@@ -90,13 +102,32 @@ __global__ void __launch_bounds__(256) keystream_kernel(const __grid_constant__ 
 
 // ---- One-trajectory route (see traj_records in common.cuh; the warp and chunk bodies are in chaos_dev.cuh).
 
-// K2t: the records of six frames per warp, one chain per frame (lane 4c + v: variable v of frame
-// 6 blockIdx.x + c).
-__global__ void __launch_bounds__(32) trajectory_kernel(const __grid_constant__ Batch b) {
-    const int lane = threadIdx.x;
-    const uint32_t f = blockIdx.x * kChainsPerWarp + (lane >> 2);
-    const bool active = (lane >> 2) < kChainsPerWarp && f < b.count;
-    trajectory_warp(active ? &b.f[f] : nullptr, b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, lane);
+// Warps per CTA of the kernels whose chains step on the integer pipes: one to each of the SM's sub-partitions.
+// With one-warp CTAs two chains may meet on a sub-partition while others are free, which costs a pipeline of many
+// launches: the clip pipeline (720 trajectories in flight) 11.3k frames/s, 13.1k with four warps per CTA, and a
+// single launch the same either way (6.29 ms for 30 frames).  Two frames to a warp, 6.55 ms and 13.8k, were left:
+// marked steps of either frame hold both up.
+constexpr uint32_t kIntWarps = 4;
+
+// One worker pair per warp, its two chains on the integer pipes (lorenz_int.cuh).
+__global__ void __launch_bounds__(32 * kIntWarps, 1) keystream_pair_kernel(const __grid_constant__ Batch b) {
+    const uint32_t task = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const uint32_t f = task / b.n, pg = task % b.n;
+    if (f >= b.count) return;
+    keystream_warp<1>(b.f[f], b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, pg, threadIdx.x & 31, &b.tab);
+}
+// Most worker pairs of a launch of it: one warp per sub-partition of the GPU (152 SMs).  Up to there a pair's
+// latency is the launch's (32 pairs of a 720p frame: 3.29 ms against 4.23 ms for the binary64 kernel; 3.41 ms with
+// four pairs per CTA, whose byte stores meet in one SM, so that CTAs have one warp while the SMs last); beyond, its
+// one pair per warp would cost more issue slots than the binary64 kernel's three have pipe time.
+constexpr uint32_t kPairLaunch = 608;
+
+// K2t: the records of one frame per warp, its chain in lanes 0..3.
+__global__ void __launch_bounds__(32 * kIntWarps, 1) trajectory_kernel(const __grid_constant__ Batch b) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t f = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (f >= b.count) return;
+    trajectory_warp(lane < 4 ? &b.f[f] : nullptr, b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, b.tab, lane);
 }
 
 // K2e: D and B of every frame from its records.  CTA (x, f) takes worker slice i = x / cps of frame f and
@@ -126,6 +157,64 @@ int g_ks_route = FHD_KS_ROUTE_TRAJECTORY;
 
 }  // namespace
 
+// Error bounds of the integer step's shadows (lorenz_int.cuh), unscaled, for |x|, |y| < 32, |z| < 64, |w| < 256
+// and |gamma| < 2: interval arithmetic over the stages with u = 2^-24 the rounding unit of a float.  A state's
+// shadow is off by less than 2^-23 of its range; a stage's by that, plus c times the error of k, plus roundings.
+// All bounds are taken over the four stages and widened by a quarter.
+IntStepTab int_step_tab(double h) {
+    IntStepTab t{};
+    t.c[0] = h / 2.0;
+    t.c[1] = h;
+    t.c[2] = h / 6.0;
+    // the step constants' shift range (c_place in 0..31 for every k and acc) and 26 significant low bits; beyond
+    // h = 0.04 the bounds mark too many steps
+    t.ok = h >= 0.0008 && h <= 0.04;
+    for (double c : t.c) {
+        unsigned long long bits;
+        std::memcpy(&bits, &c, sizeof bits);
+        if ((bits & 0x3ffffffull) == 0) t.ok = 0;
+    }
+    if (!t.ok) return t;
+    const double u = 0x1p-24, lim[4] = {32, 32, 64, 256}, g = 2.0, beta = 8.0 / 3.0;
+    const double X = lim[0], Y = lim[1], Z = lim[2], W = lim[3];
+    const double kmax[4] = {10 * (X + Y) + W, 28 * X + Y + X * Z, beta * Z + X * Y, g * W + Y * Z};
+    double es[4], e[4], acc[4] = {}, amax[4] = {}, d1[4] = {}, d2[4] = {}, et[4] = {};
+    for (int v = 0; v < 4; ++v) es[v] = e[v] = lim[v] * 0x1p-23;
+    for (int st = 0; st < 4; ++st) {
+        const double t1[4] = {e[0] + e[1] + u * (X + Y), 28 * (e[0] + u * X), beta * e[2] + 2 * u * beta * Z,
+                              g * e[3] + 2 * u * g * W};
+        const double t2[4] = {10 * t1[0] + 20 * u * (X + Y), t1[1] + e[1] + u * (56 * X + 2 * Y), t1[2], t1[3]};
+        const double q[4] = {e[3] + 2 * u * W, X * e[2] + Z * e[0] + e[0] * e[2] + 2 * u * X * Z,
+                             X * e[1] + Y * e[0] + e[0] * e[1] + 2 * u * X * Y,
+                             Y * e[2] + Z * e[1] + e[1] * e[2] + 2 * u * Y * Z};
+        const double f = st == 1 || st == 2 ? 2.0 : 1.0, c = st == 2 ? h : st == 3 ? h / 6.0 : h / 2.0;
+        for (int v = 0; v < 4; ++v) {
+            const double k = t2[v] + q[v] + u * kmax[v];
+            d1[v] = std::max(d1[v], t1[v]);
+            d2[v] = std::max(d2[v], t2[v] + 3 * u * kmax[v]);
+            amax[v] += f * kmax[v];
+            acc[v] += f * k + u * amax[v];
+            e[v] = es[v] + c * (st == 3 ? acc[v] : k) + 2 * u * c * (st == 3 ? amax[v] : kmax[v]) + u * lim[v];
+            et[v] = std::max(et[v], e[v]);
+        }
+    }
+    const int grid_kappa[4] = {kKappaXYZ, kKappaXYZ, kKappaXYZ, kKappaW};
+    const int sA[4] = {-1, 0, 0, 1}, sB[4] = {3, 2, 1, 2};
+    for (int v = 0; v < 4; ++v) {
+        const double scale = 1.1 * std::ldexp(1.0, grid_kappa[v]);
+        t.d1[v] = (float)(scale * d1[v]);
+        t.d2[v] = (float)(scale * d2[v]);
+        t.dt[v] = (float)(scale * (es[v] + u * lim[v] + 2 * u * h * kmax[v]));
+        t.limit[v] = (float)std::ldexp(lim[v], grid_kappa[v]);
+        // |A~| qA + |B~| qB in this lane's scale: A~, B~ carry their own lanes' scales
+        const double eA = sA[v] < 0 ? 0.0 : et[sA[v]], eB = et[sB[v]], lB = lim[sB[v]], lA = sA[v] < 0 ? 1.0 : lim[sA[v]];
+        const int kA = sA[v] < 0 ? kKappaXYZ : grid_kappa[sA[v]], kB = grid_kappa[sB[v]];
+        t.qA[v] = (float)(scale * (eB + eA * eB / lA + 2 * u * lB) / std::ldexp(1.0, kA));
+        t.qB[v] = (float)(scale * (eA + 2 * u * lA) / std::ldexp(1.0, kB));
+    }
+    return t;
+}
+
 int set_keystream_route(int route) {
     if (route != FHD_KS_ROUTE_TRAJECTORY && route != FHD_KS_ROUTE_PAIRS) return -1;
     const int old = g_ks_route;
@@ -142,7 +231,8 @@ cudaError_t launch_trajectory_keystream(const Batch &b, cudaStream_t s) {
         const uint64_t nb = (b.f[k].N + b.n - 1) / b.n;
         nb_max = nb > nb_max ? nb : nb_max;
     }
-    trajectory_kernel<<<(b.count + kChainsPerWarp - 1) / kChainsPerWarp, 32, 0, s>>>(b);
+    const uint32_t wpc = b.count < kIntWarps ? b.count : kIntWarps;
+    trajectory_kernel<<<(b.count + wpc - 1) / wpc, 32 * wpc, 0, s>>>(b);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -166,7 +256,8 @@ cudaError_t launch_master(const Batch &b, StreamState *states, unsigned *status,
 cudaError_t launch_master_raw(double *state5, const uint8_t *H, uint32_t n, double hstep, const uint32_t u[4],
                               double *IR, unsigned *status, cudaStream_t s) {
     Rk4 c{hstep, hstep / 2.0, hstep / 6.0};   // host arithmetic: IEEE round-to-nearest
-    master_raw_kernel<<<1, 32, 0, s>>>(state5, H, n, c, make_uint4(u[0], u[1], u[2], u[3]), IR, status);
+    master_raw_kernel<<<1, 32, 0, s>>>(state5, H, n, c, int_step_tab(hstep), make_uint4(u[0], u[1], u[2], u[3]), IR,
+                                       status);
     note_launch();
     return cudaGetLastError();
 }
@@ -188,6 +279,12 @@ cudaError_t launch_keystream(const Batch &b, cudaStream_t s, bool dense, uint32_
             keystream_kernel<4, true><<<(warps + k - 1) / k, 32 * k, smem, s>>>(b);
         else
             keystream_kernel<4><<<(warps + k - 1) / k, 32 * k, smem, s>>>(b);
+        note_launch();
+        return cudaGetLastError();
+    }
+    if (k == 1 && smem == 0 && b.count * b.n <= kPairLaunch) {
+        const uint32_t pairs = b.count * b.n, wpc = (pairs + 151) / 152;   // 1..4: an SM's pairs in one CTA
+        keystream_pair_kernel<<<(pairs + wpc - 1) / wpc, 32 * wpc, 0, s>>>(b);
         note_launch();
         return cudaGetLastError();
     }

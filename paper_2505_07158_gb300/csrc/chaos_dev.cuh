@@ -5,6 +5,7 @@
 #include "binary64_int.cuh"
 #include "bounds.cuh"
 #include "common.cuh"
+#include "lorenz_int.cuh"
 #include "sha256_core.cuh"
 
 namespace fhd {
@@ -198,6 +199,62 @@ __device__ __forceinline__ void rk4_step_lanes8_int(double &s, const LaneRole8 &
     }
 }
 
+__device__ __forceinline__ unsigned long long low48(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0xffffffffffffull;
+}
+
+// One binary64 step for Chains' marked steps, out of line: the hot loop keeps its registers and its code small.
+__device__ __noinline__ double binary64_redo(double s, int lane, double gamma, double h, double hh, double h6) {
+    const LaneRole role = lane_role(lane, gamma);
+    rk4_step_lanes(s, role, Rk4{h, hh, h6});
+    return s;
+}
+
+// The chains of a warp in the six-chain layout (lane 4c + v: variable v of chain c; lanes 24..31 the constants of
+// rk4_step_lanes), stepped on the integer pipes; a step that the integer form marks is done again in binary64.
+// live: lanes of the warp's chains.  All 32 lanes call every member together.  Where usable() is false (a step
+// size or gamma outside the integer form's range) the caller steps in binary64.
+struct Chains {
+    double s;        // the state, where `fresh`
+    IntVar q;        // the state in the integer step's form
+    IntLane L;
+    double gamma;
+    Rk4 c;
+    bool live, fresh;
+
+    static __device__ __forceinline__ bool usable(bool live, double gamma, const IntStepTab &tab) {
+        return tab.ok != 0 && __all_sync(0xffffffffu, !live || int_gamma_ok(gamma));
+    }
+    __device__ __forceinline__ void init(int lane, bool live_, double gamma_, const Rk4 &c_, const IntStepTab &tab) {
+        gamma = gamma_;
+        c = c_;
+        live = live_;
+        L = int_lane(tab, lane, gamma);
+    }
+    // The state becomes lane_init of this lane's value.
+    __device__ __forceinline__ void load(double v) {
+        s = v;
+        fresh = true;
+        int_from_double(q, s, L);
+    }
+    __device__ __forceinline__ void step(int lane) {
+        const IntVar q0 = q;
+        const bool bad = int_step(q, L);
+        const bool redo = __any_sync(0xffffffffu, bad && live);
+        if (redo) {
+            if (!fresh && lane < 4 * kChainsPerWarp) s = int_to_double(q0, L);
+            s = binary64_redo(s, lane, gamma, c.h, c.hh, c.h6);
+            int_from_double(q, s, L);
+        }
+        fresh = redo;
+    }
+    __device__ __forceinline__ double value() const { return fresh ? s : int_to_double(q, L); }
+    // The six low mantissa bytes of the value.
+    __device__ __forceinline__ unsigned long long mantissa48() const {
+        return fresh ? low48(s) : int_significand(q) & 0xffffffffffffull;
+    }
+};
+
 // Sec. II-A, Fig. 1a: reconstruct one initial condition from 8 digest bytes
 // (two for the integer part mod u, six for the 48-bit fraction), v by
 // magnitude; non-finite or |v| >= 2^52 contributes 0 and 0.
@@ -221,13 +278,25 @@ __device__ __forceinline__ double reconstruct(double v, const uint8_t *hb, uint3
 __device__ __forceinline__ bool finite(double x) { return isfinite(x); }
 
 // Reconstruct from (state, H), run LHCS_m 2n steps writing IR.  The chain
-// lives in lanes 0..3 of the warp (lane = variable); s is this lane's value.
-__device__ void master_frame(double &s, int lane, const LaneRole &role, const uint8_t *H_smem, const uint32_t *u,
-                             uint32_t n, const Rk4 &c, double *IR) {
+// lives in lanes 0..3 of the warp (lane = variable); s is this lane's value (the other lanes': lane_init).
+__device__ __forceinline__ void master_frame(double &s, int lane, Chains &ch, bool use_int, const uint8_t *H_smem,
+                                             const uint32_t *u, uint32_t n, double *IR) {
     if (lane < 4) s = reconstruct(s, H_smem + 8 * lane, u[lane]);
     __syncwarp();
+    if (use_int) {
+        ch.load(s);
+        for (uint32_t t = 0; t < 2 * n; ++t) {
+            ch.step(lane);
+            if (lane < 4) {
+                s = ch.value();
+                if (FHD_IN(4 * t + lane, 8ull * n, kSiteMasterIR)) IR[4 * t + lane] = s;
+            }
+        }
+        return;
+    }
+    const LaneRole role = lane_role(lane, ch.gamma);
     for (uint32_t t = 0; t < 2 * n; ++t) {
-        rk4_step_lanes(s, role, c);
+        rk4_step_lanes(s, role, ch.c);
         if (lane < 4 && FHD_IN(4 * t + lane, 8ull * n, kSiteMasterIR)) IR[4 * t + lane] = s;
     }
 }
@@ -274,9 +343,8 @@ __device__ __forceinline__ WorkerSlice worker_slice(uint64_t LD, uint64_t LB, ui
 // Bytes of one step: the pair's XOR of the 6 low mantissa bytes of each
 // variable; this lane writes its half (3 bytes) at stream position pos0 on.
 // dlim and blim are the bytes of D and of B from Dbytes and Bp on (range checks of checked builds).
-__device__ __forceinline__ void emit_bytes(double s, bool active, uint64_t pos0, uint64_t need, uint64_t ndb, int half,
+__device__ __forceinline__ void emit_bytes48(unsigned long long mine, bool active, uint64_t pos0, uint64_t need, uint64_t ndb, int half,
                                            uint8_t *Dbytes, uint8_t *Bp, uint64_t dlim, uint64_t blim) {
-    const unsigned long long mine = (unsigned long long)__double_as_longlong(s) & 0xffffffffffffull;
     const unsigned long long x = mine ^ __shfl_xor_sync(0xffffffffu, mine, 4);
     if (active && pos0 < need) {
 #pragma unroll
@@ -292,11 +360,18 @@ __device__ __forceinline__ void emit_bytes(double s, bool active, uint64_t pos0,
     }
 }
 
+__device__ __forceinline__ void emit_bytes(double s, bool active, uint64_t pos0, uint64_t need, uint64_t ndb, int half,
+                                           uint8_t *Dbytes, uint8_t *Bp, uint64_t dlim, uint64_t blim) {
+    emit_bytes48(low48(s), active, pos0, need, ndb, half, Dbytes, Bp, dlim, blim);
+}
+
 // Worker pairs pg * kPairs .. pg * kPairs + kPairs - 1 of frame fd (Algorithm 2), run by one warp (lane = its
 // lane): lane 4c + v holds variable v of chain c, chains 2q and 2q + 1 are pair q, so the partner of a lane
 // is lane ^ 4.  Every warp of the frame runs the frame's uniform trip count (its longest slice).
+// kPairs = 1 steps its two chains through Chains (tab: its bounds); the others take no tab.
 template <int kPairs, bool kInt = false>
-__device__ void keystream_warp(const FrameDesc &fd, uint32_t n, const Rk4 &c, uint32_t pg, int lane) {
+__device__ void keystream_warp(const FrameDesc &fd, uint32_t n, const Rk4 &c, uint32_t pg, int lane,
+                               const IntStepTab *tab = nullptr) {
     const int v = lane & 3, ch = lane >> 2;
     const uint32_t p = pg * kPairs + (ch >> 1);
     const bool active = lane < 8 * kPairs && p < n;
@@ -315,7 +390,24 @@ __device__ void keystream_warp(const FrameDesc &fd, uint32_t n, const Rk4 &c, ui
     const uint64_t ndb = 2 * ws.nd;
     const uint64_t dlim = 2 * LD - 2 * ws.d0, blim = LB - ws.b0;
     const int half = (ch & 1) * 3;
-    if (kPairs == kPairsPerWarp) {
+    if constexpr (kPairs == 1) {
+        double s = lane_init(lane, chain_value);
+        if (Chains::usable(active, fd.gamma, *tab)) {
+            Chains cc;
+            cc.init(lane, active, fd.gamma, c, *tab);
+            cc.load(s);
+            for (uint64_t t = 0; t < T; ++t) {
+                cc.step(lane);
+                emit_bytes48(cc.mantissa48(), active, 24 * t + 6 * v, need, ndb, half, Dbytes, Bp, dlim, blim);
+            }
+        } else {
+            const LaneRole role = lane_role(lane, fd.gamma);
+            for (uint64_t t = 0; t < T; ++t) {
+                rk4_step_lanes(s, role, c);
+                emit_bytes(s, active, 24 * t + 6 * v, need, ndb, half, Dbytes, Bp, dlim, blim);
+            }
+        }
+    } else if (kPairs == kPairsPerWarp) {
         const LaneRole role = lane_role(lane, fd.gamma);
         double s = lane_init(lane, chain_value);
         for (uint64_t t = 0; t < T; ++t) {
@@ -340,31 +432,27 @@ __device__ void keystream_warp(const FrameDesc &fd, uint32_t n, const Rk4 &c, ui
 
 // ---- One-trajectory keystream route (traj_records in common.cuh).
 
-__device__ __forceinline__ unsigned long long low48(double x) {
-    return (unsigned long long)__double_as_longlong(x) & 0xffffffffffffull;
-}
-
 // The records of one frame per chain of the warp, in the six-chain layout of LHCS_m (lane 4c + v holds
 // variable v of chain c; lanes 24..31 hold the constants).  fd: this lane's frame (the four lanes of a chain
-// share it), nullptr where the chain has none.  Steps k = 1, 2, ... take the state from s_k to s_{k+1}:
+// share it), nullptr where the chain has none (the launches give a warp one chain).  Steps k = 1, 2, ... take the state from s_k to s_{k+1}:
 // while k < 2n it is LHCS_m's iterate IR[k], read back, and from k = 2n on one RK4 step.  After step k >= 2
-// the warp writes record k - 2 = (s_k, s_{k+1}): the 48-bit XOR of each variable's two bit patterns (its six
-// low mantissa bytes) is packed with the next variable's by one shuffle, and lanes v = 0, 1, 2 store the
-// record's three 64-bit words.  A chain is strictly sequential, so its time is the number of steps times the
-// step's latency (27 binary64 instructions back to back, plus the hand-offs); the warp runs to its longest
-// frame.  All 32 lanes call it together.
-__device__ void trajectory_warp(const FrameDesc *fd, uint32_t n, const Rk4 &c, int lane) {
+// the warp writes record k - 2 = (s_k, s_{k+1}): each lane the 48-bit XOR of its variable's two bit patterns
+// (the six low mantissa bytes) as three 16-bit words, which needs no exchange between the lanes: a shuffle that
+// reads a fresh binary64 result, as the earlier packing into 64-bit words did, cost ~100 cycles a step.  A chain
+// is strictly sequential, so its time is the number of steps times the step's latency; the warp runs to its
+// longest frame.  All 32 lanes call it together.
+__device__ void trajectory_warp(const FrameDesc *fd, uint32_t n, const Rk4 &c, const IntStepTab &tab, int lane) {
     const int v = lane & 3;
     const bool active = fd != nullptr && lane < 4 * kChainsPerWarp;
     uint64_t R = 0;
     double gamma = 0.0;
     const double *IR = nullptr;
-    uint64_t *rec = nullptr;
+    uint8_t *rec = nullptr;
     if (active) {
         R = traj_records((uint64_t)fd->C * (fd->h + fd->w), fd->N, n);
         gamma = fd->gamma;
         IR = fd->IR;
-        rec = reinterpret_cast<uint64_t *>(fd->T);
+        rec = fd->T + 6 * v;
     }
     unsigned long long Rmax = R;
 #pragma unroll
@@ -372,22 +460,37 @@ __device__ void trajectory_warp(const FrameDesc *fd, uint32_t n, const Rk4 &c, i
         const unsigned long long t = __shfl_xor_sync(0xffffffffu, Rmax, o);
         Rmax = t > Rmax ? t : Rmax;
     }
-    const LaneRole role = lane_role(lane, gamma);
     double s = lane_init(lane, active && FHD_IN(v, 8ull * n, kSiteTrajIR) ? __ldcg(IR + v) : 0.0);   // s_1
     unsigned long long prev = low48(s);
-    for (uint64_t k = 1; k <= Rmax + 1; ++k) {
-        if (k < 2ull * n) {   // s_{k+1} = IR[k] (uniform over the warp)
-            if (active && FHD_IN(4 * k + v, 8ull * n, kSiteTrajIR)) s = __ldcg(IR + 4 * k + v);
-        } else {
-            rk4_step_lanes(s, role, c);
+    auto record = [&](uint64_t r, unsigned long long cur) {
+        if (active && r < R && FHD_IN(3 * r + 2, 3 * R, kSiteTrajRecord)) {
+            const unsigned long long x = prev ^ cur;
+            uint16_t *p = reinterpret_cast<uint16_t *>(rec + 24 * r);
+            p[0] = (uint16_t)x;
+            p[1] = (uint16_t)(x >> 16);
+            p[2] = (uint16_t)(x >> 32);
         }
-        const unsigned long long cur = low48(s);
-        const unsigned long long x = prev ^ cur;
-        const unsigned long long nx = __shfl_down_sync(0xffffffffu, x, 1);
-        const uint64_t r = k - 2;
-        if (k >= 2 && active && v < 3 && r < R && FHD_IN(3 * r + v, 3 * R, kSiteTrajRecord))
-            rec[3 * r + v] = (x >> (16 * v)) | (nx << (48 - 16 * v));
         prev = cur;
+    };
+    const uint64_t kend = Rmax + 1, kread = 2ull * n - 1 < kend ? 2ull * n - 1 : kend;
+    for (uint64_t k = 1; k <= kread; ++k) {   // s_{k+1} = IR[k] (uniform over the warp)
+        if (active && FHD_IN(4 * k + v, 8ull * n, kSiteTrajIR)) s = __ldcg(IR + 4 * k + v);
+        record(k - 2, low48(s));   // k = 1: r wraps, no record
+    }
+    if (Chains::usable(active, gamma, tab)) {
+        Chains ch;
+        ch.init(lane, active, gamma, c, tab);
+        ch.load(s);
+        for (uint64_t k = kread + 1; k <= kend; ++k) {
+            ch.step(lane);
+            record(k - 2, ch.mantissa48());
+        }
+    } else {
+        const LaneRole role = lane_role(lane, gamma);
+        for (uint64_t k = kread + 1; k <= kend; ++k) {
+            rk4_step_lanes(s, role, c);
+            record(k - 2, low48(s));
+        }
     }
 }
 
@@ -471,7 +574,9 @@ __device__ void master_stream(const BatchT &b, uint32_t g, StreamState *states, 
     const uint32_t slot = b.f[b.order[first]].slot;
     StreamState *st = states + slot;
     const double gamma = b.f[b.order[first]].gamma;
-    const LaneRole role = lane_role(lane, gamma);
+    Chains ch;
+    ch.init(lane, lane < 4, gamma, c, b.tab);
+    const bool use_int = Chains::usable(lane < 4, gamma, b.tab);
     double s = lane_init(lane, lane < 4 ? st->v[lane] : 0.0);
     uint32_t done = 0;
     for (uint32_t k = first; k < last; ++k) {
@@ -505,7 +610,7 @@ __device__ void master_stream(const BatchT &b, uint32_t g, StreamState *states, 
             }
             __syncwarp();
         }
-        master_frame(s, lane, role, H, b.u, b.n, c, fd.IR);
+        master_frame(s, lane, ch, use_int, H, b.u, b.n, fd.IR);
         __syncwarp();
         ++done;
         after(b.order[k]);

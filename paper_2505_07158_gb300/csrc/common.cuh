@@ -11,6 +11,17 @@ namespace fhd {
 // (well under the 32 KB parameter limit of sm_70+ with CUDA 12.1+).
 constexpr int kMaxBatch = 256;
 
+// Bounds and constants of the integer RK4 step for one step size (lorenz_int.cuh), by variable (x, y, z, w) in
+// the scale of its shadows: bounds of the shadows' errors (T1 or T, T2, tin's own part, and A B as
+// |A| qA + |B| qB) and the variable's range.
+struct IntStepTab {
+    float d1[4], d2[4], dt[4], qA[4], qB[4], limit[4];
+    double c[3];   // h/2, h, h/6
+    uint32_t ok;   // 0: the step size is outside the integer step's range
+    uint32_t pad;
+};
+IntStepTab int_step_tab(double h);   // chaos.cu
+
 // Per-frame launch descriptor.  All pointers are device pointers.
 struct FrameDesc {
     const uint8_t *src;
@@ -43,6 +54,7 @@ struct Batch {
     uint32_t encrypt;         // 1: this batch encrypts (LHCS_m masks the digest), 0: decrypts (unmasks)
     uint32_t int_mix;         // eight-chain worker warps per 8 that step on the integer pipes (0..8)
     double hstep, hhalf, hsixth;   // RK4 step h, h/2 and h/6 (rounded once, on the host)
+    IntStepTab tab;
     uint32_t u[4];            // reconstruction bounds
     uint16_t order[kMaxBatch];          // frame indices grouped by stream, in call order
     uint16_t group_begin[kMaxBatch + 1];
@@ -76,6 +88,7 @@ struct PSide {
     uint32_t count, n, groups;
     uint32_t digest_mode, digest_masked, encrypt;
     double hstep, hhalf, hsixth;
+    IntStepTab tab;
     uint32_t u[4];
     uint16_t order[kPMax];
     uint16_t group_begin[kPMax + 1];
@@ -224,7 +237,7 @@ cudaError_t launch_master_raw(double *state5, const uint8_t *H, uint32_t n, doub
 cudaError_t launch_keystream(const Batch &b, cudaStream_t s, bool dense = false, uint32_t warps_per_cta = 1,
                              uint32_t smem = 0);
 cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s);
-// The one-trajectory route: every frame's records (one chain per frame, six frames per warp), then D and B
+// The one-trajectory route: every frame's records (one chain and one warp per frame), then D and B
 // from them.  Each frame needs f.T (traj_bytes).
 cudaError_t launch_trajectory_keystream(const Batch &b, cudaStream_t s);
 int set_keystream_route(int route);   // FHD_KS_ROUTE_TRAJECTORY or FHD_KS_ROUTE_PAIRS; -1 on a bad value

@@ -178,8 +178,9 @@ __device__ __noinline__ void keystream_task(const FrameDesc &fd, uint32_t n, con
 }
 
 // One-trajectory route: the frame's trajectory on chain 0 of the warp (lanes 0..3).
-__device__ __noinline__ void trajectory_task(const FrameDesc &fd, uint32_t n, const Rk4 &c, int lane) {
-    trajectory_warp(lane < 4 ? &fd : nullptr, n, c, lane);
+__device__ __noinline__ void trajectory_task(const FrameDesc &fd, uint32_t n, const Rk4 &c, const IntStepTab &tab,
+                                             int lane) {
+    trajectory_warp(lane < 4 ? &fd : nullptr, n, c, tab, lane);
 }
 
 // Emission task idx of a frame (one-trajectory route): B bytes [idx kEmitTaskBytes, (idx + 1) kEmitTaskBytes)
@@ -254,7 +255,7 @@ __device__ void chain_worker(const PLaunch &L, uint8_t *H) {
                 continue;
             const PSide &S = L.s[side];
             if (wait(&L.cnt->master_done[side][f], 1u)) {
-                if (L.traj) trajectory_task(S.f[f], S.n, Rk4{S.hstep, S.hhalf, S.hsixth}, lane);
+                if (L.traj) trajectory_task(S.f[f], S.n, Rk4{S.hstep, S.hhalf, S.hsixth}, S.tab, lane);
                 else keystream_task(S.f[f], S.n, Rk4{S.hstep, S.hhalf, S.hsixth}, pg, lane);
             }
             __threadfence();
