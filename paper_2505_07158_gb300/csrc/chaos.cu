@@ -109,17 +109,16 @@ __global__ void __launch_bounds__(256) keystream_kernel(const __grid_constant__ 
 // marked steps of either frame hold both up.
 constexpr uint32_t kIntWarps = 4;
 
-// One worker pair per warp, its two chains on the integer pipes (lorenz_int.cuh).
-__global__ void __launch_bounds__(32 * kIntWarps, 1) keystream_pair_kernel(const __grid_constant__ Batch b) {
-    const uint32_t task = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint32_t f = task / b.n, pg = task % b.n;
+// One worker pair per one-warp CTA, its two chains on the integer pipes (lorenz_int.cuh).
+__global__ void __launch_bounds__(32, 1) keystream_pair_kernel(const __grid_constant__ Batch b) {
+    const uint32_t f = blockIdx.x / b.n, pg = blockIdx.x % b.n;
     if (f >= b.count) return;
-    keystream_warp<1>(b.f[f], b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, pg, threadIdx.x & 31, &b.tab);
+    keystream_warp<1>(b.f[f], b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, pg, threadIdx.x, &b.tab);
 }
 // Most worker pairs of a launch of it: one warp per sub-partition of the GPU (152 SMs).  Up to there a pair's
-// latency is the launch's (32 pairs of a 720p frame: 3.29 ms against 4.23 ms for the binary64 kernel; 3.41 ms with
-// four pairs per CTA, whose byte stores meet in one SM, so that CTAs have one warp while the SMs last); beyond, its
-// one pair per warp would cost more issue slots than the binary64 kernel's three have pipe time.
+// latency is the launch's (32 pairs of a 720p frame: 3.25 ms against 4.23 ms for the binary64 kernel; 3.36 ms with
+// four pairs per CTA; 608 pairs of 27 KB: 1.03 ms and 1.06 ms); beyond, its one pair per warp would cost more issue slots than the binary64 kernel's three
+// have pipe time.
 constexpr uint32_t kPairLaunch = 608;
 
 // K2t: the records of one frame per warp, its chain in lanes 0..3.
@@ -283,8 +282,7 @@ cudaError_t launch_keystream(const Batch &b, cudaStream_t s, bool dense, uint32_
         return cudaGetLastError();
     }
     if (k == 1 && smem == 0 && b.count * b.n <= kPairLaunch) {
-        const uint32_t pairs = b.count * b.n, wpc = (pairs + 151) / 152;   // 1..4: an SM's pairs in one CTA
-        keystream_pair_kernel<<<(pairs + wpc - 1) / wpc, 32 * wpc, 0, s>>>(b);
+        keystream_pair_kernel<<<b.count * b.n, 32, 0, s>>>(b);
         note_launch();
         return cudaGetLastError();
     }
