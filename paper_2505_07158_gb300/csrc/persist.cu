@@ -4,7 +4,7 @@
 // same frames through a sender's and a receiver's streams), runs as one kernel of one CTA per SM.  Each CTA
 // carries three kinds of workers, each pulling tasks from its own device queue (an atomic counter over a
 // task order fixed by the launch descriptor):
-//   * warps 0 and 1: a digest pipeline (the producer/consumer SHA-256 of Sec. II-A, 32 sub-frame messages
+//   * warps 0, 1 and 2: a digest pipeline (the producer/consumer SHA-256 of Sec. II-A, 32 sub-frame messages
 //     per task, largest frames first); the pipeline that completes a frame's messages folds (Algorithm 1)
 //     or tree-hashes them into the frame digest and publishes it;
 //   * warps 2, 3 and 5: chain workers, one on each of sub-partitions 1-3, so that a chain has its
@@ -35,22 +35,24 @@
 namespace fhd {
 namespace {
 
-// Warp roles by SM sub-partition (warp w runs on sub-partition w mod 4): the digest pipeline's consumer
-// (warp 0) and producer (warp 1) on sub-partitions 0 and 1; the chain workers (warps 2, 3 and 5) on
-// sub-partitions 2, 3 and 1, one each -- in a digest CTA they start only after its pipeline (below), so
-// the integer-bound digest rounds never share an issue port with a binary64 chain; warps 4 and 6-15 form
+// Warp roles by SM sub-partition (warp w runs on sub-partition w mod 4): the digest pipeline's consumers
+// (warps 0 and 1) and producer (warp 2, a chain worker afterwards) on sub-partitions 0, 1 and 2; the chain
+// workers (warps 2, 3 and 5) on sub-partitions 2, 3 and 1, one each -- in a digest CTA they start only after
+// its pipeline (below), so the digest rounds never share an issue port with a chain; warps 4 and 6-15 form
 // the permutation group.  Four warps per sub-partition leave each of them 128 registers (a
 // sub-partition's register file holds 16K).
 constexpr int kPWarps = 16;
 constexpr int kPThreads = 32 * kPWarps;
-constexpr int kShaConsumer = 0, kShaProducer = 1;
 constexpr int kChainWarps = 3;   // warps 2, 3, 5
 constexpr int kMemThreads = 32 * (kPWarps - 2 - kChainWarps);
 __device__ __forceinline__ int chain_index(uint32_t warp) { return warp == 2 ? 0 : warp == 3 ? 1 : warp == 5 ? 2 : -1; }
 __device__ __forceinline__ uint32_t mem_index(uint32_t warp) { return warp == 4 ? 0 : warp - 5; }   // warps 4, 6..15
 constexpr unsigned kBarSha = 1, kBarMem = 2;
-constexpr size_t kPFixedSmem = sizeof(ShaSmem) + 32 * kChainWarps + 64 + 16;   // + broadcast slots, flag
+// Shared memory: digests of the chain workers, broadcast slots and flag; then the digest pipeline's and, from
+// kPMemOffset, the permutation group's, which overlap: in a CTA with a pipeline the group starts after it.
+constexpr size_t kPHeadSmem = 32 * kChainWarps + 64 + 16, kPMemOffset = 24752;
 constexpr size_t kPSmemLimit = 232448;
+static_assert(kPHeadSmem % 16 == 0 && kPMemOffset % 16 == 0 && kPHeadSmem <= kPMemOffset, "16-byte aligned parts");
 
 __device__ __forceinline__ unsigned long long globaltimer() {
     unsigned long long t;
@@ -107,7 +109,7 @@ __device__ __forceinline__ uint32_t segment(const uint32_t *a, uint32_t m, uint3
 __device__ __noinline__ void digest_task(const PLaunch &L, uint32_t task, uint32_t rtid, ShaSmem &sm) {
     const PSide &S = L.s[0];
     const uint32_t n = S.n;
-    sha_pipeline(
+    sha_pipeline<true>(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             if (!FHD_IN(m / n, S.count, kSiteShaDigest) || !FHD_IN(L.prio[m / n], S.count, kSitePersistTask))
                 return false;
@@ -124,20 +126,20 @@ __device__ __noinline__ void digest_task(const PLaunch &L, uint32_t task, uint32
         S.count * n, task, rtid, kBarSha, sm);
 }
 
-// ---- digest pipeline (warps 0-1)
+// ---- digest pipeline (warps 0-2)
 __device__ void digest_worker(const PLaunch &L, ShaSmem &sm, unsigned *slot) {
-    const uint32_t rtid = (threadIdx.x >> 5) == kShaConsumer ? (threadIdx.x & 31) : 32 + (threadIdx.x & 31);
+    const uint32_t rtid = threadIdx.x;
     const PSide &S = L.s[0];
     const uint32_t n = S.n, nmsg = S.count * n;
     for (;;) {
         if (rtid == 0) slot[0] = ld_acquire(&L.cnt->abort) ? L.sha_units : atomicAdd(&L.cnt->sha_next, 1u);
-        bar_sync(kBarSha, 64);
+        bar_sync(kBarSha, kShaThreads<true>);
         const uint32_t task = slot[0];
-        bar_sync(kBarSha, 64);
+        bar_sync(kBarSha, kShaThreads<true>);
         if (task >= L.sha_units) return;
         digest_task(L, task, rtid, sm);
         __threadfence();
-        bar_sync(kBarSha, 64);
+        bar_sync(kBarSha, kShaThreads<true>);
         if (rtid == 0) {
             // the frames this task's messages belong to: count them in, and the task that completes a
             // frame forms its digest
@@ -383,11 +385,11 @@ __device__ bool wait_digest_cta(const PLaunch &L, volatile unsigned *flag) {
 // 16 warps x 128 registers fill the SM's register file: one CTA per SM, and no spills in the task bodies.
 __global__ void __maxnreg__(128) persistent_kernel(const __grid_constant__ PLaunch L) {
     extern __shared__ __align__(16) uint8_t smem[];
-    ShaSmem &sm = *reinterpret_cast<ShaSmem *>(smem);
-    uint8_t *H = smem + sizeof(ShaSmem);
+    uint8_t *H = smem;
+    ShaSmem &sm = *reinterpret_cast<ShaSmem *>(smem + kPHeadSmem);
     unsigned *slot = reinterpret_cast<unsigned *>(H + 32 * kChainWarps);   // [0] digest, [4..7] permutation,
     volatile unsigned *digest_cta_done = slot + 8;                          // [8] this CTA's digests finished
-    uint8_t *mem = smem + kPFixedSmem;
+    uint8_t *mem = smem + kPMemOffset;
     const uint32_t warp = threadIdx.x >> 5;
     const bool digest_cta = blockIdx.x < L.sha_units;
     if (threadIdx.x == 0) {
@@ -395,15 +397,16 @@ __global__ void __maxnreg__(128) persistent_kernel(const __grid_constant__ PLaun
         if (blockIdx.x == 0) L.cnt->t0 = globaltimer();
     }
     __syncthreads();
-    if (warp == kShaConsumer || warp == kShaProducer) {
-        if (digest_cta) {
-            digest_worker(L, sm, slot);
-            if (threadIdx.x == 0) {
-                __threadfence_block();
-                *digest_cta_done = 1u;
-            }
+    if (digest_cta && threadIdx.x < kShaThreads<true>) {
+        digest_worker(L, sm, slot);
+        if (threadIdx.x == 0) {
+            __threadfence_block();
+            *digest_cta_done = 1u;
         }
-    } else if (chain_index(warp) >= 0) {
+        __syncwarp();
+    }
+    if (warp < 2) return;
+    if (chain_index(warp) >= 0) {
         if (wait_digest_cta(L, digest_cta_done)) chain_worker(L, H + 32 * chain_index(warp));
     } else {
         if (wait_digest_cta(L, digest_cta_done)) mem_worker(L, mem, slot + 4);
@@ -412,13 +415,13 @@ __global__ void __maxnreg__(128) persistent_kernel(const __grid_constant__ PLaun
 
 }  // namespace
 
-size_t persistent_mem_smem_limit() { return kPSmemLimit - kPFixedSmem; }
+size_t persistent_mem_smem_limit() { return kPSmemLimit - kPMemOffset; }
 
 cudaError_t launch_persistent(const PLaunch &L, size_t mem_smem, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t smem = kPFixedSmem + mem_smem;
+    const size_t smem = std::max(kPHeadSmem + sizeof(ShaSmem), kPMemOffset + mem_smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPSmemLimit);
     if (e != cudaSuccess) return e;

@@ -7,14 +7,16 @@
 //
 // GPU mapping: a message is inherently sequential, and with n = 32 a frame has
 // only 32 of them, so the time of one message is the time of the frame.  Each
-// message therefore gets two threads in two warps of one CTA: a producer lane
-// brings the 64-byte blocks in (cp.async into a four-block shared-memory ring
-// when the message start is 16-byte aligned, byte loads otherwise; an L2
-// prefetch runs eight blocks ahead), expands the message schedule and stores
-// W[t] + K[t] into a double-buffered shared-memory ring; the consumer lane
-// runs only the 64 compression rounds of the previous block.  The two warps
-// meet at one named barrier per block.  Rotations are funnel shifts, the
-// three-input boolean functions map onto LOP3.
+// message therefore gets threads in two roles of one CTA: a producer lane
+// brings the 64-byte blocks in (cp.async of the 16-byte pieces of a message
+// at any alignment into a four-block shared-memory ring; an L2 prefetch runs
+// eight blocks ahead), expands the message schedule and stores W[t] + K[t]
+// into a double-buffered shared-memory ring; one or two consumer lanes run
+// only the 64 compression rounds of the previous block.  The warps meet at
+// one named barrier per block.  Rotations are funnel shifts, the three-input
+// boolean functions map onto LOP3.  16 frames of 720p: 1.33 ms with one
+// consumer lane and every sum on the integer pipe, 1.19 ms with the off-chain
+// sums on the multiplier's and 16-byte ring accesses, 1.07 ms with two lanes.
 #include <mutex>
 
 #include "common.cuh"
@@ -24,10 +26,11 @@ namespace fhd {
 namespace {
 
 // Sub-frame messages of a batch: message m is sub-frame m % n of frame m / n.
-__global__ void __launch_bounds__(64) sha_subframes_kernel(const __grid_constant__ Batch b) {
+template <bool kSplit>
+__global__ void __launch_bounds__(kShaThreads<kSplit>) sha_subframes_kernel(const __grid_constant__ Batch b) {
     __shared__ ShaSmem sm;
     const uint32_t n = b.n;
-    sha_pipeline(
+    sha_pipeline<kSplit>(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             if (!FHD_IN(m / n, b.count, kSiteShaDigest)) return false;
             const FrameDesc &fd = b.f[m / n];
@@ -44,10 +47,11 @@ __global__ void __launch_bounds__(64) sha_subframes_kernel(const __grid_constant
 }
 
 // `count` buffers of nbytes laid end to end, n sub-frames each.
-__global__ void __launch_bounds__(64) sha_plain_kernel(const uint8_t *data, uint64_t nbytes, uint32_t n,
-                                                       uint32_t count, uint8_t *part) {
+template <bool kSplit>
+__global__ void __launch_bounds__(kShaThreads<kSplit>) sha_plain_kernel(const uint8_t *data, uint64_t nbytes, uint32_t n,
+                                                                uint32_t count, uint8_t *part) {
     __shared__ ShaSmem sm;
-    sha_pipeline(
+    sha_pipeline<kSplit>(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             const uint32_t k = m / n, i = m % n;
             const uint64_t lo = (uint64_t)(((unsigned __int128)nbytes * i) / n);
@@ -63,10 +67,11 @@ __global__ void __launch_bounds__(64) sha_plain_kernel(const uint8_t *data, uint
 
 // Sub-frame messages of the decrypted frames (dst) of a batch, for the
 // receiver-side check; digests go to part (n per frame).
-__global__ void __launch_bounds__(64) sha_dst_kernel(const __grid_constant__ Batch b) {
+template <bool kSplit>
+__global__ void __launch_bounds__(kShaThreads<kSplit>) sha_dst_kernel(const __grid_constant__ Batch b) {
     __shared__ ShaSmem sm;
     const uint32_t n = b.n;
-    sha_pipeline(
+    sha_pipeline<kSplit>(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             if (!FHD_IN(m / n, b.count, kSiteShaDigest)) return false;
             const FrameDesc &fd = b.f[m / n];
@@ -180,10 +185,20 @@ cudaError_t noalloc_scratch(uint8_t **out) {
     return cudaSuccess;
 }
 
+// Split messages while every pipeline has an SM to itself: 16 pipelines (16 frames of 720p) take 1.07 ms split
+// and 1.19 ms unsplit.  Where two share one, the two split consumer warps of the one meet those of the other on the same
+// sub-partitions, whose integer pipe one of them already fills: 256 pipelines (1080p) take 4.30 ms split and
+// 2.76 ms unsplit.
+static bool split_messages(uint32_t units) { return units <= 152; }
+
 cudaError_t launch_sha_subframes(const Batch &b, cudaStream_t s) {
     const uint32_t msgs = b.count * b.n;
     if (!msgs) return cudaSuccess;
-    sha_subframes_kernel<<<(msgs + kMsgPerCta - 1) / kMsgPerCta, 64, 0, s>>>(b);
+    const uint32_t units = (msgs + kMsgPerCta - 1) / kMsgPerCta;
+    if (split_messages(units))
+        sha_subframes_kernel<true><<<units, kShaThreads<true>, 0, s>>>(b);
+    else
+        sha_subframes_kernel<false><<<units, kShaThreads<false>, 0, s>>>(b);
     note_launch();
     return cudaGetLastError();
 }
@@ -191,7 +206,11 @@ cudaError_t launch_sha_subframes(const Batch &b, cudaStream_t s) {
 cudaError_t launch_verify(const Batch &b, uint8_t *ok, cudaStream_t s) {
     const uint32_t msgs = b.count * b.n;
     if (!msgs) return cudaSuccess;
-    sha_dst_kernel<<<(msgs + kMsgPerCta - 1) / kMsgPerCta, 64, 0, s>>>(b);
+    const uint32_t units = (msgs + kMsgPerCta - 1) / kMsgPerCta;
+    if (split_messages(units))
+        sha_dst_kernel<true><<<units, kShaThreads<true>, 0, s>>>(b);
+    else
+        sha_dst_kernel<false><<<units, kShaThreads<false>, 0, s>>>(b);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -204,7 +223,11 @@ cudaError_t launch_sha_plain(const uint8_t *data, uint64_t nbytes, uint32_t n, u
                              cudaStream_t s) {
     const uint32_t msgs = count * n;
     if (!msgs) return cudaSuccess;
-    sha_plain_kernel<<<(msgs + kMsgPerCta - 1) / kMsgPerCta, 64, 0, s>>>(data, nbytes, n, count, part);
+    const uint32_t units = (msgs + kMsgPerCta - 1) / kMsgPerCta;
+    if (split_messages(units))
+        sha_plain_kernel<true><<<units, kShaThreads<true>, 0, s>>>(data, nbytes, n, count, part);
+    else
+        sha_plain_kernel<false><<<units, kShaThreads<false>, 0, s>>>(data, nbytes, n, count, part);
     note_launch();
     return cudaGetLastError();
 }
