@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(32, 1) master_raw_kernel(double *state5, const
     const double gamma = state5[4];
     Chains ch;
     ch.init(lane, lane < 4, gamma, c, tab);
-    const bool use_int = Chains::usable(lane < 4, gamma, tab);
+    const bool use_int = Chains::usable(lane < 4, lane, gamma, tab);
     double s = lane_init(lane, lane < 4 ? state5[lane] : 0.0);
     master_frame(s, lane, ch, use_int, H, u, n, IR);
     if (lane < 4) {
@@ -116,9 +116,9 @@ __global__ void __launch_bounds__(32, 1) keystream_pair_kernel(const __grid_cons
     keystream_warp<1>(b.f[f], b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, pg, threadIdx.x, &b.tab);
 }
 // Most worker pairs of a launch of it: one warp per sub-partition of the GPU (152 SMs).  Up to there a pair's
-// latency is the launch's (32 pairs of a 720p frame: 3.25 ms against 4.23 ms for the binary64 kernel; 3.36 ms with
-// four pairs per CTA; 608 pairs of 27 KB: 1.03 ms and 1.06 ms); beyond, its one pair per warp would cost more issue slots than the binary64 kernel's three
-// have pipe time.
+// latency is the launch's (32 pairs of a 720p frame: 2.91 ms against 4.23 ms for the binary64 kernel; four pairs
+// per CTA took 3 % longer, with 608 pairs too); beyond, its one pair per warp would cost more issue slots than the
+// binary64 kernel's three have pipe time.
 constexpr uint32_t kPairLaunch = 608;
 
 // K2t: the records of one frame per warp, its chain in lanes 0..3.
@@ -165,49 +165,52 @@ IntStepTab int_step_tab(double h) {
     t.c[0] = h / 2.0;
     t.c[1] = h;
     t.c[2] = h / 6.0;
-    // the step constants' shift range (c_place in 0..31 for every k and acc) and 26 significant low bits; beyond
+    // the step constants' shift range (c_place in 0..31 for every k and acc) and a one among their low 19 bits; beyond
     // h = 0.04 the bounds mark too many steps
     t.ok = h >= 0.0008 && h <= 0.04;
     for (double c : t.c) {
         unsigned long long bits;
         std::memcpy(&bits, &c, sizeof bits);
-        if ((bits & 0x3ffffffull) == 0) t.ok = 0;
+        if ((bits & 0x7ffffull) == 0) t.ok = 0;
     }
     if (!t.ok) return t;
-    const double u = 0x1p-24, lim[4] = {32, 32, 64, 256}, g = 2.0, beta = 8.0 / 3.0;
+    // ranges: just beyond the attractor's, each within the power of two that the shifts allow
+    const double u = 0x1p-24, lim[4] = {28, 30, 50, 216}, end[4] = {32, 32, 64, 256}, g = 2.0, beta = 8.0 / 3.0;
     const double X = lim[0], Y = lim[1], Z = lim[2], W = lim[3];
     const double kmax[4] = {10 * (X + Y) + W, 28 * X + Y + X * Z, beta * Z + X * Y, g * W + Y * Z};
-    double es[4], e[4], acc[4] = {}, amax[4] = {}, d1[4] = {}, d2[4] = {}, et[4] = {};
-    for (int v = 0; v < 4; ++v) es[v] = e[v] = lim[v] * 0x1p-23;
+    double es[4], e[4], acc[4] = {}, amax[4] = {}, d1[4] = {}, d2[4] = {}, dk[4] = {}, et[4] = {};
+    for (int v = 0; v < 4; ++v) es[v] = e[v] = end[v] * 0x1p-23;
     for (int st = 0; st < 4; ++st) {
-        const double t1[4] = {e[0] + e[1] + u * (X + Y), 28 * (e[0] + u * X), beta * e[2] + 2 * u * beta * Z,
-                              g * e[3] + 2 * u * g * W};
+        const double t1[4] = {e[0] + e[1] + u * (X + Y), 28 * (e[0] + u * X), beta * e[2] + (0x1p-21 + u * beta) * Z,
+                              g * e[3] + (0x1p-22 + u * g) * W};
         const double t2[4] = {10 * t1[0] + 20 * u * (X + Y), t1[1] + e[1] + u * (56 * X + 2 * Y), t1[2], t1[3]};
-        const double q[4] = {e[3] + 2 * u * W, X * e[2] + Z * e[0] + e[0] * e[2] + 2 * u * X * Z,
+        const double q[4] = {e[3] + (0x1p-22 + 3 * u) * W, X * e[2] + Z * e[0] + e[0] * e[2] + 2 * u * X * Z,
                              X * e[1] + Y * e[0] + e[0] * e[1] + 2 * u * X * Y,
                              Y * e[2] + Z * e[1] + e[1] * e[2] + 2 * u * Y * Z};
         const double f = st == 1 || st == 2 ? 2.0 : 1.0, c = st == 2 ? h : st == 3 ? h / 6.0 : h / 2.0;
         for (int v = 0; v < 4; ++v) {
             const double k = t2[v] + q[v] + u * kmax[v];
             d1[v] = std::max(d1[v], t1[v]);
-            d2[v] = std::max(d2[v], t2[v] + 3 * u * kmax[v]);
+            d2[v] = std::max(d2[v], t2[v]);
+            dk[v] = std::max(dk[v], t2[v] + 3 * u * kmax[v]);
             amax[v] += f * kmax[v];
             acc[v] += f * k + u * amax[v];
             e[v] = es[v] + c * (st == 3 ? acc[v] : k) + 2 * u * c * (st == 3 ? amax[v] : kmax[v]) + u * lim[v];
             et[v] = std::max(et[v], e[v]);
         }
     }
-    const int grid_kappa[4] = {kKappaXYZ, kKappaXYZ, kKappaXYZ, kKappaW};
+    const int grid_kappa[4] = {int_kappa(0), int_kappa(1), int_kappa(2), int_kappa(3)};
     const int sA[4] = {-1, 0, 0, 1}, sB[4] = {3, 2, 1, 2};
     for (int v = 0; v < 4; ++v) {
         const double scale = 1.1 * std::ldexp(1.0, grid_kappa[v]);
         t.d1[v] = (float)(scale * d1[v]);
         t.d2[v] = (float)(scale * d2[v]);
+        t.dk[v] = (float)(scale * dk[v]);
         t.dt[v] = (float)(scale * (es[v] + u * lim[v] + 2 * u * h * kmax[v]));
         t.limit[v] = (float)std::ldexp(lim[v], grid_kappa[v]);
         // |A~| qA + |B~| qB in this lane's scale: A~, B~ carry their own lanes' scales
-        const double eA = sA[v] < 0 ? 0.0 : et[sA[v]], eB = et[sB[v]], lB = lim[sB[v]], lA = sA[v] < 0 ? 1.0 : lim[sA[v]];
-        const int kA = sA[v] < 0 ? kKappaXYZ : grid_kappa[sA[v]], kB = grid_kappa[sB[v]];
+        const double eA = sA[v] < 0 ? 0x1p-22 : et[sA[v]], eB = et[sB[v]], lB = lim[sB[v]], lA = sA[v] < 0 ? 1.0 : lim[sA[v]];
+        const int kA = sA[v] < 0 ? int_kappa(3) : grid_kappa[sA[v]], kB = grid_kappa[sB[v]];
         t.qA[v] = (float)(scale * (eB + eA * eB / lA + 2 * u * lB) / std::ldexp(1.0, kA));
         t.qB[v] = (float)(scale * (eA + 2 * u * lA) / std::ldexp(1.0, kB));
     }

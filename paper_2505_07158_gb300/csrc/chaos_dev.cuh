@@ -210,49 +210,73 @@ __device__ __noinline__ double binary64_redo(double s, int lane, double gamma, d
     return s;
 }
 
-// The chains of a warp in the six-chain layout (lane 4c + v: variable v of chain c; lanes 24..31 the constants of
+// Up to two chains of a warp in the six-chain layout (lane 4c + v: variable v of chain c; lanes 24..31 the constants of
 // rk4_step_lanes), stepped on the integer pipes; a step that the integer form marks is done again in binary64.
 // live: lanes of the warp's chains.  All 32 lanes call every member together.  Where usable() is false (a step
 // size or gamma outside the integer form's range) the caller steps in binary64.
 struct Chains {
     double s;        // the state, where `fresh`
     IntVar q;        // the state in the integer step's form
+    IntOthers o;     // and its exchange: its shuffles run while the step's marks are voted on
     IntLane L;
     double gamma;
     Rk4 c;
+    unsigned long long m48;   // the six low mantissa bytes of the state
     bool live, fresh;
 
-    static __device__ __forceinline__ bool usable(bool live, double gamma, const IntStepTab &tab) {
-        return tab.ok != 0 && __all_sync(0xffffffffu, !live || int_gamma_ok(gamma));
+    static __device__ __forceinline__ bool usable(bool live, int lane, double gamma, const IntStepTab &tab) {
+        return tab.ok != 0 && __all_sync(0xffffffffu, !live || (lane < 4 * kIntChains && int_gamma_ok(gamma)));
     }
     __device__ __forceinline__ void init(int lane, bool live_, double gamma_, const Rk4 &c_, const IntStepTab &tab) {
         gamma = gamma_;
         c = c_;
         live = live_;
-        L = int_lane(tab, lane, gamma);
+        L = int_lane(tab, lane);
+        int_constants(q, L, lane, gamma);
     }
     // The state becomes lane_init of this lane's value.
-    __device__ __forceinline__ void load(double v) {
+    __device__ __forceinline__ void load(double v, int lane) {
         s = v;
         fresh = true;
-        int_from_double(q, s, L);
+        m48 = low48(s);
+        if (lane < 4 * kIntChains) int_from_double(q, s, L);
+        o = int_exchange(q, L);
+    }
+    // One step; false where it is marked, and then redo(q0) has to follow, q0 being the state before it.
+    __device__ __forceinline__ bool try_step() {
+        const bool bad = int_step(q, o, L);
+        o = int_exchange(q, L);
+        m48 = int_significand(q) & 0xffffffffffffull;
+        return !__any_sync(0xffffffffu, bad && live);
+    }
+    __device__ __forceinline__ void redo(const IntVar &q0, int lane) {
+        if (!fresh && lane < 4 * kIntChains) s = int_to_double(q0, L);
+        load(binary64_redo(s, lane, gamma, c.h, c.hh, c.h6), lane);
+    }
+    // `count` steps, each after before_step(m48, i), i its number.  The loop without the redo's call in it keeps its
+    // registers in place: 5.22 ms for the records of a 1080p frame, 5.34 ms with a call of step() per turn.
+    template <class F>
+    __device__ __forceinline__ void steps(uint64_t count, int lane, F &&before_step) {
+        for (uint64_t i = 0; i < count;) {
+            IntVar q0;
+            bool good = true;
+            while (i < count) {
+                before_step(m48, i);
+                ++i;
+                q0 = q;
+                good = try_step();
+                if (!good) break;
+                fresh = false;
+            }
+            if (!good) redo(q0, lane);
+        }
     }
     __device__ __forceinline__ void step(int lane) {
         const IntVar q0 = q;
-        const bool bad = int_step(q, L);
-        const bool redo = __any_sync(0xffffffffu, bad && live);
-        if (redo) {
-            if (!fresh && lane < 4 * kChainsPerWarp) s = int_to_double(q0, L);
-            s = binary64_redo(s, lane, gamma, c.h, c.hh, c.h6);
-            int_from_double(q, s, L);
-        }
-        fresh = redo;
+        if (try_step()) fresh = false;
+        else redo(q0, lane);
     }
     __device__ __forceinline__ double value() const { return fresh ? s : int_to_double(q, L); }
-    // The six low mantissa bytes of the value.
-    __device__ __forceinline__ unsigned long long mantissa48() const {
-        return fresh ? low48(s) : int_significand(q) & 0xffffffffffffull;
-    }
 };
 
 // Sec. II-A, Fig. 1a: reconstruct one initial condition from 8 digest bytes
@@ -284,7 +308,7 @@ __device__ __forceinline__ void master_frame(double &s, int lane, Chains &ch, bo
     if (lane < 4) s = reconstruct(s, H_smem + 8 * lane, u[lane]);
     __syncwarp();
     if (use_int) {
-        ch.load(s);
+        ch.load(s, lane);
         for (uint32_t t = 0; t < 2 * n; ++t) {
             ch.step(lane);
             if (lane < 4) {
@@ -392,14 +416,14 @@ __device__ void keystream_warp(const FrameDesc &fd, uint32_t n, const Rk4 &c, ui
     const int half = (ch & 1) * 3;
     if constexpr (kPairs == 1) {
         double s = lane_init(lane, chain_value);
-        if (Chains::usable(active, fd.gamma, *tab)) {
+        if (Chains::usable(active, lane, fd.gamma, *tab)) {
             Chains cc;
             cc.init(lane, active, fd.gamma, c, *tab);
-            cc.load(s);
-            for (uint64_t t = 0; t < T; ++t) {
-                cc.step(lane);
-                emit_bytes48(cc.mantissa48(), active, 24 * t + 6 * v, need, ndb, half, Dbytes, Bp, dlim, blim);
-            }
+            cc.load(s, lane);
+            cc.steps(T, lane, [&](unsigned long long m48, uint64_t t) {   // a step's bytes beside the next step's instructions
+                if (t) emit_bytes48(m48, active, 24 * (t - 1) + 6 * v, need, ndb, half, Dbytes, Bp, dlim, blim);
+            });
+            if (T) emit_bytes48(cc.m48, active, 24 * (T - 1) + 6 * v, need, ndb, half, Dbytes, Bp, dlim, blim);
         } else {
             const LaneRole role = lane_role(lane, fd.gamma);
             for (uint64_t t = 0; t < T; ++t) {
@@ -462,34 +486,39 @@ __device__ void trajectory_warp(const FrameDesc *fd, uint32_t n, const Rk4 &c, c
     }
     double s = lane_init(lane, active && FHD_IN(v, 8ull * n, kSiteTrajIR) ? __ldcg(IR + v) : 0.0);   // s_1
     unsigned long long prev = low48(s);
-    auto record = [&](uint64_t r, unsigned long long cur) {
-        if (active && r < R && FHD_IN(3 * r + 2, 3 * R, kSiteTrajRecord)) {
+    uint8_t *const rec_end = rec + 24 * R;
+    auto record = [&](unsigned long long cur) {   // the next record
+        if (active && rec < rec_end && FHD_IN((uint64_t)(rec_end - rec) / 8, 3 * R + 1, kSiteTrajRecord)) {
             const unsigned long long x = prev ^ cur;
-            uint16_t *p = reinterpret_cast<uint16_t *>(rec + 24 * r);
+            uint16_t *p = reinterpret_cast<uint16_t *>(rec);
             p[0] = (uint16_t)x;
             p[1] = (uint16_t)(x >> 16);
             p[2] = (uint16_t)(x >> 32);
         }
         prev = cur;
+        rec += 24;
     };
     const uint64_t kend = Rmax + 1, kread = 2ull * n - 1 < kend ? 2ull * n - 1 : kend;
     for (uint64_t k = 1; k <= kread; ++k) {   // s_{k+1} = IR[k] (uniform over the warp)
         if (active && FHD_IN(4 * k + v, 8ull * n, kSiteTrajIR)) s = __ldcg(IR + 4 * k + v);
-        record(k - 2, low48(s));   // k = 1: r wraps, no record
+        if (k > 1) record(low48(s));
+        else prev = low48(s);
     }
-    if (Chains::usable(active, gamma, tab)) {
+    if (Chains::usable(active, lane, gamma, tab)) {
         Chains ch;
         ch.init(lane, active, gamma, c, tab);
-        ch.load(s);
-        for (uint64_t k = kread + 1; k <= kend; ++k) {
+        ch.load(s, lane);
+        // a record is written beside the next step's instructions
+        if (kread < kend) {
             ch.step(lane);
-            record(k - 2, ch.mantissa48());
+            ch.steps(kend - kread - 1, lane, [&](unsigned long long m48, uint64_t) { record(m48); });
+            record(ch.m48);
         }
     } else {
         const LaneRole role = lane_role(lane, gamma);
         for (uint64_t k = kread + 1; k <= kend; ++k) {
             rk4_step_lanes(s, role, c);
-            record(k - 2, low48(s));
+            record(low48(s));
         }
     }
 }
@@ -576,7 +605,7 @@ __device__ void master_stream(const BatchT &b, uint32_t g, StreamState *states, 
     const double gamma = b.f[b.order[first]].gamma;
     Chains ch;
     ch.init(lane, lane < 4, gamma, c, b.tab);
-    const bool use_int = Chains::usable(lane < 4, gamma, b.tab);
+    const bool use_int = Chains::usable(lane < 4, lane, gamma, b.tab);
     double s = lane_init(lane, lane < 4 ? st->v[lane] : 0.0);
     uint32_t done = 0;
     for (uint32_t k = first; k < last; ++k) {

@@ -15,7 +15,7 @@ constexpr int kMaxBatch = 256;
 // the scale of its shadows: bounds of the shadows' errors (T1 or T, T2, tin's own part, and A B as
 // |A| qA + |B| qB) and the variable's range.
 struct IntStepTab {
-    float d1[4], d2[4], dt[4], qA[4], qB[4], limit[4];
+    float d1[4], d2[4], dk[4], dt[4], qA[4], qB[4], limit[4];
     double c[3];   // h/2, h, h/6
     uint32_t ok;   // 0: the step size is outside the integer step's range
     uint32_t pad;

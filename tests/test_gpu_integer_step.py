@@ -104,3 +104,18 @@ def test_trajectories_of_a_batch_with_other_gammas(count):
         E_ref, H_ref = ref.encrypt(F)
         assert np.array_equal(host(E), E_ref) and bytes(host(H)) == H_ref
     c.close()
+
+
+def test_states_at_the_edges_of_each_grid():
+    """Each variable round its range and round the smallest magnitudes of the grids, in both chains of a pair."""
+    g = si.rng(17)
+    base = _attractor(g, -0.9, 1)[0]
+    rows = []
+    for v, lim in enumerate((28.0, 30.0, 50.0, 216.0)):
+        for x in (lim, 2.0 ** -9, 2.0 ** -10, 2.0 ** -11, 2.0 ** -12, 2.0 ** -13, 1.0 + 2.0 ** -20, 1.0 + 2.0 ** -33):
+            for y in (np.nextafter(x, 0), x, np.nextafter(x, 1e9)):
+                for sign in (1.0, -1.0):
+                    s = base.copy()
+                    s[v] = sign * y
+                    rows.append(s)
+    _pairs(np.array(rows), -0.9123, len(rows) // 2, shape=(64, 80, 3))
