@@ -255,33 +255,71 @@ __global__ void __launch_bounds__(kStatThreads) corr_kernel(const uint8_t *frame
 // histograms in shared memory and writes each channel's entropy; a second
 // kernel takes the mean over the k blocks in block order (a fixed summation
 // order, so the result does not depend on scheduling).
+//
+// Read row by row, a block was 44 round trips to memory, and its 768 terms
+// z log2 z, ~30 binary64 instructions each, held the binary64 pipes for most
+// of the rest.  The bytes are now read kLoads to a thread at a time whatever
+// the row, and a term is computed once for each count that occurs up to 256
+// (the counts of a block are small: the largest of the 900 noise blocks of
+// 44 x 44 in 30 frames is under 32, one warp's work).  The five statistics of that clip: 349 -> 292 us.
+template <int C>
 __global__ void __launch_bounds__(kStatThreads) block_entropy_kernel(const uint8_t *frames, uint32_t h, uint32_t w,
-                                                                     uint32_t C, const uint32_t *blocks, uint32_t k,
-                                                                     uint32_t bs, double *ent, unsigned *status) {
-    __shared__ uint32_t hist[4][256];
+                                                                     const uint32_t *blocks, uint32_t k, uint32_t bs,
+                                                                     double *ent, unsigned *status) {
+    constexpr int kLoads = 8;
+    __shared__ uint32_t hist[C][256];
+    __shared__ double term[256];   // of count z in term[z - 1]
+    __shared__ uint32_t largest;
     const uint32_t f = blockIdx.x / k, q = blockIdx.x % k;
     const uint8_t *F = frames + (uint64_t)f * h * w * C;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t r0 = blocks[2 * ((uint64_t)f * k + q)], c0 = blocks[2 * ((uint64_t)f * k + q) + 1];
-    const bool inside = r0 + bs <= h && c0 + bs <= w;
-    for (uint32_t t = threadIdx.x; t < 4 * 256; t += blockDim.x) (&hist[0][0])[t] = 0;
+    const bool inside = r0 <= h - bs && c0 <= w - bs;   // bs <= h, w
+    for (uint32_t t = threadIdx.x; t < C * 256; t += kStatThreads) (&hist[0][0])[t] = 0;
+    if (threadIdx.x == 0) largest = 0;
     __syncthreads();
     if (inside) {
-        for (uint32_t i = 0; i < bs; ++i) {
-            const uint8_t *row = F + ((uint64_t)(r0 + i) * w + c0) * C;
-            for (uint32_t t = threadIdx.x; t < bs * C; t += blockDim.x)
-                if (FHD_IN(((uint64_t)(r0 + i) * w + c0) * C + t, (uint64_t)h * w * C, kSiteStats))
-                    atomicAdd(&hist[t % C][row[t]], 1u);
+        const uint32_t row = bs * C, down = kStatThreads / row, along = kStatThreads % row;
+        uint32_t i = threadIdx.x / row, t = threadIdx.x % row;
+        while (i < bs) {
+            uint8_t v[kLoads];
+            uint32_t c[kLoads];
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u) {
+                const uint64_t at = ((uint64_t)(r0 + i) * w + c0) * C + t;
+                c[u] = C;
+                if (i < bs && FHD_IN(at, (uint64_t)h * w * C, kSiteStats)) {
+                    v[u] = __ldg(F + at);
+                    c[u] = t % C;
+                }
+                i += down;
+                t += along;
+                if (t >= row) {
+                    t -= row;
+                    ++i;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u)
+                if (c[u] < C) atomicAdd(&hist[c[u]][v[u]], 1u);
         }
     } else if (threadIdx.x == 0) {
         atomicOr(status, 1u);
     }
     __syncthreads();
-    if ((uint32_t)warp < C) {
+    uint32_t z = 0;
+#pragma unroll
+    for (int c = 0; c < C; ++c) z = max(z, hist[c][threadIdx.x]);
+    z = __reduce_max_sync(0xffffffffu, z);
+    if (lane == 0) atomicMax(&largest, z);
+    __syncthreads();
+    if (threadIdx.x < largest) term[threadIdx.x] = (double)(threadIdx.x + 1) * log2((double)(threadIdx.x + 1));
+    __syncthreads();
+    if (warp < C) {
         double e = 0.0;
         for (int i = lane; i < 256; i += 32) {
             const uint32_t z = hist[warp][i];
-            if (z) e += (double)z * log2((double)z);
+            if (z) e += z <= 256 ? term[z - 1] : (double)z * log2((double)z);
         }
         for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
         const double T = (double)bs * (double)bs;
@@ -294,6 +332,7 @@ __global__ void block_entropy_mean_kernel(const double *ent, uint32_t count, uin
     if (item >= count * C) return;
     const uint32_t f = item / C, c = item % C;
     double acc = 0.0;
+#pragma unroll 8
     for (uint32_t q = 0; q < k; ++q) acc += ent[((uint64_t)f * k + q) * C + c];
     out[item] = acc / (double)k;
 }
@@ -373,7 +412,12 @@ cudaError_t launch_stats_correlation(const uint8_t *frames, uint32_t count, uint
 cudaError_t launch_stats_local_entropy(const uint8_t *frames, uint32_t count, uint32_t h, uint32_t w, uint32_t C,
                                        const uint32_t *blocks, uint32_t k, uint32_t bs, double *ent, double *out,
                                        unsigned *status, cudaStream_t s) {
-    block_entropy_kernel<<<count * k, kStatThreads, 0, s>>>(frames, h, w, C, blocks, k, bs, ent, status);
+    switch (C) {
+        case 1: block_entropy_kernel<1><<<count * k, kStatThreads, 0, s>>>(frames, h, w, blocks, k, bs, ent, status); break;
+        case 2: block_entropy_kernel<2><<<count * k, kStatThreads, 0, s>>>(frames, h, w, blocks, k, bs, ent, status); break;
+        case 3: block_entropy_kernel<3><<<count * k, kStatThreads, 0, s>>>(frames, h, w, blocks, k, bs, ent, status); break;
+        default: block_entropy_kernel<4><<<count * k, kStatThreads, 0, s>>>(frames, h, w, blocks, k, bs, ent, status); break;
+    }
     note_launch();
     block_entropy_mean_kernel<<<(count * C + 127) / 128, 128, 0, s>>>(ent, count, C, k, out);
     note_launch();

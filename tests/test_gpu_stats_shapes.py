@@ -1,0 +1,48 @@
+"""The statistics kernels at odd sizes: frames whose rows and starts are at any alignment, every channel count, blocks
+of one pixel and of the whole frame, flat frames (one large count) and coordinates outside the frame.  Counts are exact;
+an entropy is a sum of at most 256 terms of a few roundings each, so it is within 1e-12 of the same sum in numpy."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2505_07158_gb300 as fhd
+from paper_2505_07158_gb300 import _lib
+
+pytestmark = pytest.mark.gpu
+
+
+def frames(count, h, w, c, flat=False, seed=5):
+    g = np.random.default_rng(seed)
+    a = np.full((count, h, w, c), 77, dtype=np.uint8) if flat else g.integers(0, 256, size=(count, h, w, c), dtype=np.uint8)
+    return a, torch.from_numpy(a).cuda()
+
+
+def entropy(x):
+    z = np.bincount(x.reshape(-1), minlength=256).astype(np.float64)
+    z = z[z > 0]
+    return np.log2(z.sum()) - (z * np.log2(z)).sum() / z.sum()
+
+
+@pytest.mark.parametrize("c", [1, 2, 3, 4])
+@pytest.mark.parametrize("shape,bs", [((5, 7), 1), ((5, 7), 5), ((61, 47), 3), ((61, 47), 44), ((64, 300), 64), ((300, 300), 300)])
+@pytest.mark.parametrize("flat", [False, True])
+def test_local_entropy_blocks(c, shape, bs, flat):
+    a, dev = frames(3, *shape, c, flat)
+    g = np.random.default_rng(6)
+    k = 4
+    blocks = np.stack([g.integers(0, shape[0] - bs + 1, (3, k)), g.integers(0, shape[1] - bs + 1, (3, k))], -1).astype(np.int32)
+    blocks[0, 0] = (shape[0] - bs, shape[1] - bs)
+    out, status = _lib.fhd_stats_local_entropy(dev, torch.from_numpy(blocks).cuda(), bs)
+    assert int(status) == 0
+    for f in range(3):
+        for ch in range(c):
+            ref = np.mean([entropy(a[f, r:r + bs, q:q + bs, ch]) for r, q in blocks[f]])
+            assert abs(float(out[f, ch]) - ref) < 1e-12
+
+
+@pytest.mark.parametrize("block", [(-1, 0), (0, -1), (-2 ** 31, 3), (60, 0), (0, 60)])
+def test_blocks_outside_are_reported(block):
+    _, dev = frames(1, 61, 47, 3)
+    blocks = torch.tensor([[block, (0, 0)]], dtype=torch.int32, device="cuda")
+    _, status = _lib.fhd_stats_local_entropy(dev, blocks, 3)
+    assert int(status) == 1
