@@ -46,3 +46,30 @@ def test_blocks_outside_are_reported(block):
     blocks = torch.tensor([[block, (0, 0)]], dtype=torch.int32, device="cuda")
     _, status = _lib.fhd_stats_local_entropy(dev, blocks, 3)
     assert int(status) == 1
+
+
+@pytest.mark.parametrize("c", [1, 2, 3, 4])
+@pytest.mark.parametrize("shape,npairs", [((2, 2), 1), ((5, 7), 31), ((61, 47), 1024), ((61, 47), 1025), ((64, 300), 10000),
+                                          ((300, 301), 50001)])
+def test_correlation_sums(c, shape, npairs):
+    a, dev = frames(3, *shape, c)
+    g = np.random.default_rng(8)
+    pairs = np.stack([g.integers(0, shape[0] - 1, (3, 3, npairs)), g.integers(0, shape[1] - 1, (3, 3, npairs))], -1).astype(np.int32)
+    sums, r, status = _lib.fhd_stats_correlation(dev, torch.from_numpy(pairs).cuda())
+    assert int(status) == 0
+    for f in range(3):
+        for d, (di, dj) in enumerate(((0, 1), (1, 0), (1, 1))):
+            i, j = pairs[f, d, :, 0], pairs[f, d, :, 1]
+            for ch in range(c):
+                x, y = a[f, i, j, ch].astype(np.int64), a[f, i + di, j + dj, ch].astype(np.int64)
+                assert sums[f, ch, d].tolist() == [x.sum(), y.sum(), (x * x).sum(), (y * y).sum(), (x * y).sum()]
+
+
+@pytest.mark.parametrize("pair,directions", [((-1, 0), 7), ((0, -1), 7), ((60, 0), 6), ((0, 46), 5), ((61, 0), 7), ((0, 47), 7)])
+def test_pairs_outside_are_reported(pair, directions):
+    _, dev = frames(1, 61, 47, 3)
+    for d in range(3):
+        pairs = torch.zeros((1, 3, 5, 2), dtype=torch.int32)
+        pairs[0, d, 2] = torch.tensor(pair, dtype=torch.int32)
+        _, _, status = _lib.fhd_stats_correlation(dev, pairs.cuda())
+        assert int(status) == directions >> d & 1
