@@ -12,9 +12,11 @@
 // channel is a compile-time constant (C is a template parameter); per-warp
 // shared-memory histograms, or per-thread channel sums built four bytes at a
 // time with the SIMD byte instructions, are merged with one global atomic per
-// counter and CTA, and a per-(frame, channel) warp finishes the statistic.  The correlation and local-entropy
+// counter and CTA, and a CTA per (frame, channel) finishes the statistic.  The correlation and local-entropy
 // statistics read only the sampled pairs and blocks (a few kB per frame).
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "bounds.cuh"
 #include "common.cuh"
@@ -29,47 +31,84 @@ __global__ void zero_kernel(unsigned long long *p, uint64_t n) {
     for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) p[k] = 0;
 }
 
-// Channel of byte k of the batch: frames hold whole pixels, so it is k mod C.
-// Histogram pass: CTA b covers bytes [b * chunk, (b + 1) * chunk) of the
-// batch (chunk a multiple of 16 * C that divides the frame, so a CTA stays in
-// one frame and starts on channel 0).  A thread takes groups of 16 * C bytes
-// (C 16-byte loads), in which byte q belongs to channel q mod C: the channel
-// of every byte is a compile-time constant.  The CTA's counters are
+// The streaming passes cut each frame into `cuts` runs of whole 16 * C-byte groups (the last one with the rest);
+// CTA b has run b % cuts of frame b / cuts, and so starts on channel 0.
+struct Run {
+    uint64_t begin, end;   // bytes of the batch
+    uint32_t head;         // bytes before the first 16-byte boundary
+};
+template <int C>
+__device__ __forceinline__ Run stat_run(const uint8_t *p, uint64_t frame_bytes, uint32_t cuts) {
+    const uint64_t f = blockIdx.x / cuts, j = blockIdx.x % cuts, groups = frame_bytes / (16 * C);
+    Run r;
+    r.begin = f * frame_bytes + 16 * C * (groups * j / cuts);
+    r.end = j + 1 == cuts ? (f + 1) * frame_bytes : f * frame_bytes + 16 * C * (groups * (j + 1) / cuts);
+    r.head = (uint32_t)(-reinterpret_cast<uintptr_t>(p + r.begin)) & 15;
+    return r;
+}
+
+// Runs per frame: as many as give the CTAs the GPU holds at once (`slots`) a run each, several rounds of them while a
+// run is longer than `most` bytes, fewer where it would be shorter than `least`.
+uint32_t stat_cuts(uint64_t frame_bytes, uint32_t count, uint32_t C, uint64_t slots, uint64_t least, uint64_t most) {
+    const uint64_t total = frame_bytes * count, rounds = std::max<uint64_t>(1, (total + slots * most - 1) / (slots * most));
+    uint64_t cuts = std::max<uint64_t>(1, slots * rounds / count);
+    cuts = std::min(cuts, std::max<uint64_t>(1, frame_bytes / least));
+    cuts = std::min(cuts, std::max<uint64_t>(1, 0x7fffffffull / count));   // the grid's limit
+    return (uint32_t)std::min<uint64_t>(cuts, 1u << 20);
+}
+
+// Histogram pass.  A thread takes groups of 16 * C aligned bytes (C 16-byte
+// loads) in which byte q belongs to channel (PH + q) mod C, PH the run's head
+// mod C: the channel of every byte is a compile-time constant.  The CTA's counters are
 // [channel][bin][lane]: each lane counts in its own bank, so the shared
 // atomics of a warp never conflict on a bank; at the end the 32 lane copies
 // are summed and added to the frame's global histogram.
+//
+// Bound by the shared atomics, one a byte.  The runs fill the two CTAs of 96 KB (C = 3) that an SM holds: cut at
+// divisors of the frame near 512 KB, 30 frames of 1080p made 360 CTAs for 304 places, and a frame that has no
+// such divisor one CTA, which read it byte by byte.  Those 30 frames: 71 -> 51 us.
+template <int C, int PH>
+__device__ __forceinline__ void hist_groups(const uint8_t *p, uint64_t groups, uint32_t *mine) {
+    for (uint64_t k = threadIdx.x; k < groups; k += kStatThreads) {
+        uint4 v[C];
+#pragma unroll
+        for (int m = 0; m < C; ++m) v[m] = __ldcs(reinterpret_cast<const uint4 *>(p + 16 * C * k) + m);
+#pragma unroll
+        for (int m = 0; m < C; ++m) {
+            const uint32_t wd[4] = {v[m].x, v[m].y, v[m].z, v[m].w};
+#pragma unroll
+            for (int q = 0; q < 16; ++q)
+                atomicAdd(&mine[(((PH + 16 * m + q) % C) * 256 + ((wd[q >> 2] >> (8 * (q & 3))) & 255)) * 32], 1u);
+        }
+    }
+}
+
 template <int C>
 __global__ void __launch_bounds__(kStatThreads) hist_kernel(const uint8_t *frames, uint64_t total, uint64_t frame_bytes,
-                                                            uint64_t chunk, unsigned long long *hist) {
+                                                            uint32_t cuts, unsigned long long *hist) {
     extern __shared__ uint32_t sh[];   // C * 256 * 32
     const uint32_t lane = threadIdx.x & 31;
     for (uint32_t k = threadIdx.x; k < C * 256 * 32; k += blockDim.x) sh[k] = 0;
     __syncthreads();
-    const uint64_t b0 = (uint64_t)blockIdx.x * chunk;
-    const uint64_t b1 = min(b0 + chunk, total);
+    const Run run = stat_run<C>(frames, frame_bytes, cuts);
     uint32_t *mine = sh + lane;
-    constexpr uint32_t G = 16 * C;
-    const bool vec = (reinterpret_cast<uintptr_t>(frames + b0) & 15) == 0 && (b1 - b0) % G == 0;
-    if (vec) {
-        for (uint64_t k = b0 + G * (uint64_t)threadIdx.x; k < b1; k += G * (uint64_t)blockDim.x) {
-            if (!FHD_IN(k + G - 1, total, kSiteStats)) break;
-            uint4 v[C];
-#pragma unroll
-            for (int m = 0; m < C; ++m) v[m] = __ldcs(reinterpret_cast<const uint4 *>(frames + k) + m);
-#pragma unroll
-            for (int m = 0; m < C; ++m) {
-                const uint32_t wd[4] = {v[m].x, v[m].y, v[m].z, v[m].w};
-#pragma unroll
-                for (int q = 0; q < 16; ++q)
-                    atomicAdd(&mine[(((16 * m + q) % C) * 256 + ((wd[q >> 2] >> (8 * (q & 3))) & 255)) * 32], 1u);
-            }
-        }
-    } else {
-        for (uint64_t t = b0 + threadIdx.x; t < b1; t += blockDim.x)
-            atomicAdd(&mine[((uint32_t)(t % C) * 256 + frames[t]) * 32], 1u);
+    const uint64_t length = run.end - run.begin, head = min((uint64_t)run.head, length);
+    const uint64_t groups = FHD_IN(run.end, total + 1, kSiteStats) ? (length - head) / (16 * C) : 0;
+    const uint8_t *p = frames + run.begin;
+    if (groups) switch (head % C) {
+        case 0: hist_groups<C, 0>(p + head, groups, mine); break;
+        case 1: hist_groups<C, 1 % C>(p + head, groups, mine); break;
+        case 2: hist_groups<C, 2 % C>(p + head, groups, mine); break;
+        default: hist_groups<C, 3 % C>(p + head, groups, mine); break;
+    }
+    // the head and what the groups leave
+    const uint64_t done = head + 16 * C * groups;
+    for (uint64_t t = threadIdx.x; t < length - 16 * C * groups; t += kStatThreads) {
+        const uint64_t at = t < head ? t : t - head + done;
+        if (FHD_IN(run.begin + at, total, kSiteStats)) atomicAdd(&mine[((uint32_t)(at % C) * 256 + p[at]) * 32], 1u);
     }
     __syncthreads();
-    const uint64_t f = b0 / frame_bytes;
+    const uint64_t f = run.begin / frame_bytes;
     for (uint32_t q = threadIdx.x; q < C * 256; q += blockDim.x) {
         const uint32_t *row = sh + q * 32;
         uint32_t s = 0;
@@ -79,28 +118,35 @@ __global__ void __launch_bounds__(kStatThreads) hist_kernel(const uint8_t *frame
     }
 }
 
-// One warp per (frame, channel): var(Z) (Eq. 4) = S2/256 - (S1/256)^2,
+// One CTA per (frame, channel): var(Z) (Eq. 4) = S2/256 - (S1/256)^2,
 // chi^2 (Eq. 5) = (256 S2 - N^2) / N, H (Eq. 10) = log2 N - (sum z log2 z) / N.
-__global__ void hist_finish_kernel(const unsigned long long *hist, uint32_t items, uint32_t *hist32, double *out) {
-    const uint32_t item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (item >= items) return;
-    const unsigned long long *z = hist + (uint64_t)item * 256;
+// A thread per bin: its logarithm is ~30 binary64 instructions of 64 cycles, so
+// eight of them in one lane were the kernel's time.  90 histograms: 27 -> 8 us.
+__global__ void __launch_bounds__(256) hist_finish_kernel(const unsigned long long *hist, uint32_t *hist32, double *out) {
+    __shared__ unsigned long long zs[256];
+    __shared__ double term[256];
+    const uint64_t item = blockIdx.x;
+    const uint32_t t = threadIdx.x;
+    const unsigned long long v = hist[item * 256 + t];
+    zs[t] = v;
+    term[t] = v ? (double)v * log2((double)v) : 0.0;
+    if (hist32) hist32[item * 256 + t] = (uint32_t)v;
+    __syncthreads();
+    if (t >= 32) return;
     unsigned long long s1 = 0, s2 = 0;
     double zl = 0.0;
-    for (int i = lane; i < 256; i += 32) {
-        const unsigned long long v = z[i];
-        s1 += v;
-        s2 += v * v;
-        if (v) zl += (double)v * log2((double)v);
-        if (hist32) hist32[(uint64_t)item * 256 + i] = (uint32_t)v;
+#pragma unroll
+    for (uint32_t i = t; i < 256; i += 32) {
+        s1 += zs[i];
+        s2 += zs[i] * zs[i];
+        zl += term[i];
     }
     for (int o = 16; o; o >>= 1) {
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
         s2 += __shfl_xor_sync(0xffffffffu, s2, o);
         zl += __shfl_xor_sync(0xffffffffu, zl, o);
     }
-    if (lane == 0) {
+    if (t == 0) {
         const double N = (double)s1;
         const double m1 = N / 256.0;
         out[3 * item + 0] = (double)s2 / 256.0 - m1 * m1;
@@ -118,13 +164,39 @@ __host__ __device__ constexpr uint32_t chan_mask(int m, int c) {
     return r;
 }
 
-// NPCR / UACI pass: per CTA chunk and 16 * C-byte groups as in hist_kernel.
+// NPCR / UACI pass: per CTA run and 16 * C-byte groups as in hist_kernel.
 // Four bytes at a time: __vabsdiffu4 gives |a - b| per byte, __vcmpne4 marks
 // the differing bytes, and a channel's bytes of the word are summed with
 // __dp4a through a compile-time mask.
+template <int C, int PH>
+__device__ __forceinline__ void npcr_groups(const uint8_t *a, const uint8_t *b, uint64_t groups, uint32_t (&changed)[C],
+                                            uint32_t (&diff)[C]) {
+    for (uint64_t k = threadIdx.x; k < groups; k += kStatThreads) {
+        uint4 va[C], vb[C];
+#pragma unroll
+        for (int m = 0; m < C; ++m) {
+            va[m] = __ldcs(reinterpret_cast<const uint4 *>(a + 16 * C * k) + m);
+            vb[m] = __ldcs(reinterpret_cast<const uint4 *>(b + 16 * C * k) + m);
+        }
+#pragma unroll
+        for (int m = 0; m < 4 * C; ++m) {
+            const uint32_t x = (&va[m >> 2].x)[m & 3], y = (&vb[m >> 2].x)[m & 3];
+            const uint32_t d = __vabsdiffu4(x, y);
+            const uint32_t ne = __vcmpne4(x, y) & 0x01010101u;
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                constexpr uint32_t ones = 0x01010101u;
+                const uint32_t mk = chan_mask<C>(m, (c + C - PH) % C);
+                diff[c] = __dp4a(d & mk, ones, diff[c]);
+                changed[c] = __dp4a(ne & mk, ones, changed[c]);
+            }
+        }
+    }
+}
+
 template <int C>
 __global__ void __launch_bounds__(kStatThreads) npcr_kernel(const uint8_t *a, const uint8_t *b, uint64_t total,
-                                                            uint64_t frame_bytes, uint64_t chunk,
+                                                            uint64_t frame_bytes, uint32_t cuts,
                                                             unsigned long long *acc) {
     __shared__ unsigned long long sacc[4][2];
     if (threadIdx.x < 8) sacc[threadIdx.x >> 1][threadIdx.x & 1] = 0;
@@ -132,45 +204,29 @@ __global__ void __launch_bounds__(kStatThreads) npcr_kernel(const uint8_t *a, co
     uint32_t changed[C], diff[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) changed[c] = diff[c] = 0;
-    const uint64_t b0 = (uint64_t)blockIdx.x * chunk;
-    const uint64_t b1 = min(b0 + chunk, total);
-    constexpr uint32_t G = 16 * C;
-    const bool vec = ((reinterpret_cast<uintptr_t>(a + b0) | reinterpret_cast<uintptr_t>(b + b0)) & 15) == 0 &&
-                     (b1 - b0) % G == 0;
-    if (vec) {
-        for (uint64_t k = b0 + G * (uint64_t)threadIdx.x; k < b1; k += G * (uint64_t)blockDim.x) {
-            if (!FHD_IN(k + G - 1, total, kSiteStats)) break;
-            uint4 va[C], vb[C];
+    const Run run = stat_run<C>(a, frame_bytes, cuts);
+    const uint64_t length = run.end - run.begin, head = min((uint64_t)run.head, length);
+    const bool vec = ((reinterpret_cast<uintptr_t>(a) ^ reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+    const uint64_t groups = vec && FHD_IN(run.end, total + 1, kSiteStats) ? (length - head) / (16 * C) : 0;
+    const uint8_t *pa = a + run.begin, *pb = b + run.begin;
+    if (groups) switch (head % C) {
+        case 0: npcr_groups<C, 0>(pa + head, pb + head, groups, changed, diff); break;
+        case 1: npcr_groups<C, 1 % C>(pa + head, pb + head, groups, changed, diff); break;
+        case 2: npcr_groups<C, 2 % C>(pa + head, pb + head, groups, changed, diff); break;
+        default: npcr_groups<C, 3 % C>(pa + head, pb + head, groups, changed, diff); break;
+    }
+    const uint64_t done = head + 16 * C * groups;
+    for (uint64_t t = threadIdx.x; t < length - 16 * C * groups; t += kStatThreads) {
+        const uint64_t at = t < head ? t : t - head + done;
+        if (!FHD_IN(run.begin + at, total, kSiteStats)) break;
+        const uint32_t c = (uint32_t)(at % C);
+        const int x = pa[at], y = pb[at];
 #pragma unroll
-            for (int m = 0; m < C; ++m) {
-                va[m] = __ldcs(reinterpret_cast<const uint4 *>(a + k) + m);
-                vb[m] = __ldcs(reinterpret_cast<const uint4 *>(b + k) + m);
+        for (int cc = 0; cc < C; ++cc)
+            if ((uint32_t)cc == c) {
+                changed[cc] += x != y;
+                diff[cc] += (uint32_t)abs(x - y);
             }
-#pragma unroll
-            for (int m = 0; m < 4 * C; ++m) {
-                const uint32_t x = (&va[m >> 2].x)[m & 3], y = (&vb[m >> 2].x)[m & 3];
-                const uint32_t d = __vabsdiffu4(x, y);
-                const uint32_t ne = __vcmpne4(x, y) & 0x01010101u;
-#pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    constexpr uint32_t ones = 0x01010101u;
-                    const uint32_t mk = chan_mask<C>(m, c);
-                    diff[c] = __dp4a(d & mk, ones, diff[c]);
-                    changed[c] = __dp4a(ne & mk, ones, changed[c]);
-                }
-            }
-        }
-    } else {
-        for (uint64_t t = b0 + threadIdx.x; t < b1; t += blockDim.x) {
-            const uint32_t c = (uint32_t)(t % C);
-            const int x = a[t], y = b[t];
-#pragma unroll
-            for (int cc = 0; cc < C; ++cc)
-                if ((uint32_t)cc == c) {
-                    changed[cc] += x != y;
-                    diff[cc] += (uint32_t)abs(x - y);
-                }
-        }
     }
 #pragma unroll
     for (int c = 0; c < C; ++c) {
@@ -185,7 +241,7 @@ __global__ void __launch_bounds__(kStatThreads) npcr_kernel(const uint8_t *a, co
         }
     }
     __syncthreads();
-    const uint64_t f = b0 / frame_bytes;
+    const uint64_t f = run.begin / frame_bytes;
     if (threadIdx.x < 2 * C) atomicAdd(&acc[(f * C + (threadIdx.x >> 1)) * 2 + (threadIdx.x & 1)], sacc[threadIdx.x >> 1][threadIdx.x & 1]);
 }
 
@@ -398,17 +454,6 @@ __global__ void block_entropy_mean_kernel(const double *ent, uint32_t count, uin
     out[item] = acc / (double)k;
 }
 
-// Bytes per CTA of the streaming passes: a multiple of 16 * C near `target`
-// that divides the frame, so that a CTA never spans two frames and starts on
-// channel 0; frames without such a divisor down to target/16 get one CTA each.
-uint64_t stat_chunk(uint64_t frame_bytes, uint32_t C, uint64_t target = 65536) {
-    const uint64_t unit = 16ull * C;
-    if (frame_bytes % unit != 0 || frame_bytes <= target) return frame_bytes;
-    for (uint64_t chunk = unit * (target / unit); chunk >= target / 16; chunk -= unit)
-        if (frame_bytes % chunk == 0) return chunk;
-    return frame_bytes;
-}
-
 unsigned zero_grid(uint64_t n) {
     const uint64_t g = (n + 255) / 256;
     return (unsigned)(g < 1024 ? (g ? g : 1) : 1024);
@@ -422,22 +467,23 @@ cudaError_t launch_stats_histogram(const uint8_t *frames, uint32_t count, uint64
     const uint64_t items = (uint64_t)count * C;
     zero_kernel<<<zero_grid(items * 256), 256, 0, s>>>(hist64, items * 256);
     note_launch();
-    const uint64_t chunk = stat_chunk(frame_bytes, C, 1u << 19);   // ~512 kB: amortises the 32-copy merge
-    const uint64_t ctas = (total + chunk - 1) / chunk;
     const size_t smem = (size_t)C * 256 * 32 * sizeof(uint32_t);
     cudaError_t e = cudaFuncSetAttribute(hist_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e != cudaSuccess) return e;
+    // CTAs of 32 C KB of counters and 256 threads on 152 SMs; a run of 64 KB at least, for the sum of the copies
+    const uint32_t cuts = stat_cuts(frame_bytes, count, C, 152 * std::min(8u, 227u / (32 * C + 1)), 1u << 16, 1u << 20);
+    const uint64_t ctas = (uint64_t)cuts * count;
     switch (C) {
-        case 1: hist_kernel<1><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, chunk, hist64); break;
-        case 2: hist_kernel<2><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, chunk, hist64); break;
-        case 3: hist_kernel<3><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, chunk, hist64); break;
-        default: hist_kernel<4><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, chunk, hist64); break;
+        case 1: hist_kernel<1><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        case 2: hist_kernel<2><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        case 3: hist_kernel<3><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        default: hist_kernel<4><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
     }
     note_launch();
-    hist_finish_kernel<<<(unsigned)((items + 7) / 8), 256, 0, s>>>(hist64, (uint32_t)items, hist32, out);
+    hist_finish_kernel<<<(unsigned)items, 256, 0, s>>>(hist64, hist32, out);
     note_launch();
     return cudaGetLastError();
 }
@@ -448,13 +494,14 @@ cudaError_t launch_stats_npcr(const uint8_t *a, const uint8_t *b, uint32_t count
     const uint64_t items = (uint64_t)count * C;
     zero_kernel<<<zero_grid(items * 2), 256, 0, s>>>(acc, items * 2);
     note_launch();
-    const uint64_t chunk = stat_chunk(frame_bytes, C);
-    const unsigned grid = (unsigned)((total + chunk - 1) / chunk);
+    // eight CTAs of 256 threads to an SM; runs of 64 KB where there are more than a round of them
+    const uint32_t cuts = stat_cuts(frame_bytes, count, C, 152 * 8, 1u << 13, 1u << 16);
+    const unsigned grid = cuts * count;
     switch (C) {
-        case 1: npcr_kernel<1><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, chunk, acc); break;
-        case 2: npcr_kernel<2><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, chunk, acc); break;
-        case 3: npcr_kernel<3><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, chunk, acc); break;
-        default: npcr_kernel<4><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, chunk, acc); break;
+        case 1: npcr_kernel<1><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, cuts, acc); break;
+        case 2: npcr_kernel<2><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, cuts, acc); break;
+        case 3: npcr_kernel<3><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, cuts, acc); break;
+        default: npcr_kernel<4><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, cuts, acc); break;
     }
     note_launch();
     npcr_finish_kernel<<<(unsigned)((items + 255) / 256), 256, 0, s>>>(acc, (uint32_t)items, wh, out);

@@ -73,3 +73,25 @@ def test_pairs_outside_are_reported(pair, directions):
         pairs[0, d, 2] = torch.tensor(pair, dtype=torch.int32)
         _, _, status = _lib.fhd_stats_correlation(dev, pairs.cuda())
         assert int(status) == directions >> d & 1
+
+
+@pytest.mark.parametrize("c", [1, 2, 3, 4])
+@pytest.mark.parametrize("count,h,w", [(1, 1, 1), (3, 1, 5), (2, 7, 13), (5, 61, 47), (2, 333, 517), (1, 1111, 1777), (40, 64, 64)])
+@pytest.mark.parametrize("offset,skew", [(0, 0), (1, 0), (7, 0), (0, 3)])
+def test_streaming_counts(c, count, h, w, offset, skew):
+    """Every byte counted once, from any start: histograms, changed pixels and |a - b| are exact."""
+    n = count * h * w * c
+    g = np.random.default_rng(9)
+    a, b = (g.integers(0, 256, size=n + 16, dtype=np.uint8) for _ in range(2))
+    b[::3] = a[::3]
+    da = torch.from_numpy(a).cuda()[offset:offset + n].view(count, h, w, c)
+    db = torch.from_numpy(b).cuda()[offset + skew:offset + skew + n].view(count, h, w, c)
+    a, b = a[offset:offset + n].reshape(count, h * w, c), b[offset + skew:offset + skew + n].reshape(count, h * w, c)
+    hist, _ = _lib.fhd_stats_histogram(da)
+    counts, _ = _lib.fhd_stats_npcr_uaci(da, db)
+    hist, counts = hist.cpu().numpy(), counts.cpu().numpy()
+    for f in range(count):
+        for ch in range(c):
+            x, y = a[f, :, ch].astype(np.int64), b[f, :, ch].astype(np.int64)
+            assert np.array_equal(hist[f, ch], np.bincount(x, minlength=256))
+            assert counts[f, ch].tolist() == [int((x != y).sum()), int(np.abs(x - y).sum())]
