@@ -26,6 +26,9 @@ namespace {
 
 constexpr int kStatThreads = 256;
 constexpr int kStatWarps = kStatThreads / 32;
+// Threads of a histogram CTA, whose counters leave room for two in an SM at C = 3: 32 warps for the atomics'
+// latency (30 frames of 1080p: 61 us a call, 71 with 256 threads, 61 with 1024).
+constexpr int kHistThreads = 512;
 
 __global__ void zero_kernel(unsigned long long *p, uint64_t n) {
     for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (uint64_t)gridDim.x * blockDim.x) p[k] = 0;
@@ -66,10 +69,10 @@ uint32_t stat_cuts(uint64_t frame_bytes, uint32_t count, uint32_t C, uint64_t sl
 //
 // Bound by the shared atomics, one a byte.  The runs fill the two CTAs of 96 KB (C = 3) that an SM holds: cut at
 // divisors of the frame near 512 KB, 30 frames of 1080p made 360 CTAs for 304 places, and a frame that has no
-// such divisor one CTA, which read it byte by byte.  Those 30 frames: 71 -> 51 us.
+// such divisor one CTA, which read it byte by byte.  Those 30 frames: 71 -> 42 us.
 template <int C, int PH>
 __device__ __forceinline__ void hist_groups(const uint8_t *p, uint64_t groups, uint32_t *mine) {
-    for (uint64_t k = threadIdx.x; k < groups; k += kStatThreads) {
+    for (uint64_t k = threadIdx.x; k < groups; k += kHistThreads) {
         uint4 v[C];
 #pragma unroll
         for (int m = 0; m < C; ++m) v[m] = __ldcs(reinterpret_cast<const uint4 *>(p + 16 * C * k) + m);
@@ -84,7 +87,7 @@ __device__ __forceinline__ void hist_groups(const uint8_t *p, uint64_t groups, u
 }
 
 template <int C>
-__global__ void __launch_bounds__(kStatThreads) hist_kernel(const uint8_t *frames, uint64_t total, uint64_t frame_bytes,
+__global__ void __launch_bounds__(kHistThreads) hist_kernel(const uint8_t *frames, uint64_t total, uint64_t frame_bytes,
                                                             uint32_t cuts, unsigned long long *hist) {
     extern __shared__ uint32_t sh[];   // C * 256 * 32
     const uint32_t lane = threadIdx.x & 31;
@@ -103,7 +106,7 @@ __global__ void __launch_bounds__(kStatThreads) hist_kernel(const uint8_t *frame
     }
     // the head and what the groups leave
     const uint64_t done = head + 16 * C * groups;
-    for (uint64_t t = threadIdx.x; t < length - 16 * C * groups; t += kStatThreads) {
+    for (uint64_t t = threadIdx.x; t < length - 16 * C * groups; t += kHistThreads) {
         const uint64_t at = t < head ? t : t - head + done;
         if (FHD_IN(run.begin + at, total, kSiteStats)) atomicAdd(&mine[((uint32_t)(at % C) * 256 + p[at]) * 32], 1u);
     }
@@ -473,14 +476,15 @@ cudaError_t launch_stats_histogram(const uint8_t *frames, uint32_t count, uint64
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e != cudaSuccess) return e;
-    // CTAs of 32 C KB of counters and 256 threads on 152 SMs; a run of 64 KB at least, for the sum of the copies
-    const uint32_t cuts = stat_cuts(frame_bytes, count, C, 152 * std::min(8u, 227u / (32 * C + 1)), 1u << 16, 1u << 20);
+    // CTAs of 32 C KB of counters and 512 threads, at most four of them to an SM, on 152 SMs; a run of 64 KB at least,
+    // for the sum of the copies
+    const uint32_t cuts = stat_cuts(frame_bytes, count, C, 152 * std::min(4u, 227u / (32 * C + 1)), 1u << 16, 1u << 20);
     const uint64_t ctas = (uint64_t)cuts * count;
     switch (C) {
-        case 1: hist_kernel<1><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
-        case 2: hist_kernel<2><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
-        case 3: hist_kernel<3><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
-        default: hist_kernel<4><<<(unsigned)ctas, kStatThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        case 1: hist_kernel<1><<<(unsigned)ctas, kHistThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        case 2: hist_kernel<2><<<(unsigned)ctas, kHistThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        case 3: hist_kernel<3><<<(unsigned)ctas, kHistThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
+        default: hist_kernel<4><<<(unsigned)ctas, kHistThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
     }
     note_launch();
     hist_finish_kernel<<<(unsigned)items, 256, 0, s>>>(hist64, hist32, out);
