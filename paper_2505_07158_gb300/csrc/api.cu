@@ -539,6 +539,11 @@ int run_frames(fhd_cipher *c, uint32_t count, const fhd_frame *frames, void *str
             }
         }
         uint32_t ctas = 0, rctas = 0;
+        uint64_t strips = 0;
+        for (uint32_t k = 0; k < m; ++k) {
+            const fhd_frame &f = frames[base + k];
+            strips += fhd::permute_strips(f.width, fhd::strip_width(f.height, f.width, f.channels));
+        }
         for (uint32_t k = 0; k < m; ++k) {
             const fhd_frame &f = frames[base + k];
             FrameDesc &d = b.f[k];
@@ -557,7 +562,7 @@ int run_frames(fhd_cipher *c, uint32_t count, const fhd_frame *frames, void *str
             d.B = p; p += align16(d.N);
             d.G = p; p += align16(d.N);
             d.T = p; p += align16(fhd::traj_bytes((uint64_t)d.C * (d.h + d.w), d.N, c->n));
-            d.P = fhd::strip_width(d.h, d.w, d.C);
+            d.P = fhd::launch_strip_width(d.h, d.w, d.C, strips);
             d.cta0 = ctas;
             ctas += fhd::permute_strips(d.w, d.P);
             d.RB = fhd::row_band(d.h, d.w, d.C);
@@ -1617,7 +1622,8 @@ static int permute_one(const uint8_t *src, uint8_t *dst, uint32_t height, uint32
     d.w = width;
     d.C = channels;
     d.N = N;
-    d.P = fhd::strip_width(height, width, channels);
+    d.P = fhd::launch_strip_width(height, width, channels,
+                                  fhd::permute_strips(width, fhd::strip_width(height, width, channels)));
     d.cta0 = 0;
     b.perm_ctas = fhd::permute_strips(width, d.P);
     d.RB = fhd::row_band(height, width, channels);

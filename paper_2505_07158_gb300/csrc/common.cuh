@@ -248,6 +248,7 @@ int keystream_route();
 uint32_t strip_width(uint32_t h, uint32_t w, uint32_t C);
 size_t strip_smem_bytes(uint32_t h, uint32_t P, uint32_t C);
 uint32_t permute_strips(uint32_t w, uint32_t P);
+uint32_t launch_strip_width(uint32_t h, uint32_t w, uint32_t C, uint64_t strips);
 uint32_t row_band(uint32_t h, uint32_t w, uint32_t C);
 size_t row_smem_bytes(uint32_t w, uint32_t C, uint32_t RB);
 cudaError_t permute_prepare();   // opt in to large dynamic shared memory

@@ -30,14 +30,16 @@
 namespace fhd {
 namespace {
 
-// CTA shapes.  Column pass: 512 threads at two CTAs per SM (the default) or 256 at four; row pass: 256
+// CTA shapes.  Column pass: 512 threads at two CTAs per SM (the default; 1024 where the strip leaves room for one
+// CTA) or 256 at four; row pass: 256
 // threads held to six CTAs per SM (40 registers) or 128 at twelve.  The autotuner picks per frame shape
 // (fhd_set_cta_threads); on the 30-frame 1080p clip the defaults measured 0.269 / 0.259 ms per encrypt /
 // decrypt permutation call, 256-thread column-pass CTAs 0.326 / 0.368.
+constexpr size_t kSmemPerSm = 233472, kSmemReserved = 1024;   // shared memory of an SM, and what each CTA adds
 constexpr int kStripThreads = 512;
 constexpr int kRowThreads = 256;
 template <int kT>
-constexpr int strip_ctas_per_sm() { return kT == 512 ? 2 : 4; }
+constexpr int strip_ctas_per_sm() { return kT == 1024 ? 1 : kT == 512 ? 2 : 4; }
 template <int kT>
 constexpr int row_ctas_per_sm() { return kT == 256 ? 6 : 12; }
 template <bool kRow>
@@ -50,12 +52,16 @@ __device__ __forceinline__ uint32_t find_frame(const Batch &b, uint32_t cta) {
     return lo;
 }
 
+// The second pass of a call is launched while the first still runs (launch_second) and waits here for its end.
+__device__ __forceinline__ void wait_for_first_pass() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <bool kEnc, int kT = kStripThreads>
 __global__ void __launch_bounds__(kT, strip_ctas_per_sm<kT>()) strip_kernel(const __grid_constant__ Batch b,
                                                                             uint32_t cta_base) {
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<false>(b, cta)];
+    wait_for_first_pass();
     strip_pass<kEnc>(fd, cta - fd.cta0, smem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
@@ -65,6 +71,7 @@ __global__ void __launch_bounds__(kT, row_ctas_per_sm<kT>()) row_kernel(const __
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<true>(b, cta)];
+    wait_for_first_pass();
     row_pass<kEnc>(fd, cta - fd.rcta0, smem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
@@ -244,6 +251,7 @@ __global__ void __launch_bounds__(kGatherThreads, 2) gather_encrypt_kernel(const
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<false>(b, cta)];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t h = fd.h, w = fd.w, P = fd.P;
     const uint32_t j0 = (cta - fd.cta0) * P;
     if (!FHD_IN(j0, w, kSiteGatherSmem)) return;   // a strip past the frame (the whole CTA)
@@ -387,8 +395,22 @@ uint32_t strip_width(uint32_t h, uint32_t w, uint32_t C) {
     return strip_smem_bytes(h, P, C) <= kSmemLimit ? P : 0;
 }
 
+// Strip widths of a launch whose strips at strip_width() are `strips` in all: where they would leave more than half
+// of the SMs idle, half as wide (again), down to 32 bytes of a row.  A frame by itself, both ways: 1080p 30 strips of
+// 64 pixels 62 us, 120 of 16 46 us; 1081 x 1917 (bytewise) 303 us and 172; 4K 120 strips of 32 93 us, 240 of 16
+// 101 us.
+uint32_t launch_strip_width(uint32_t h, uint32_t w, uint32_t C, uint64_t strips) {
+    for (int k = 0; k < g_overrides; ++k)
+        if (g_override_key[k][0] == h && g_override_key[k][1] == w && g_override_key[k][2] == C && g_override_P[k])
+            return strip_width(h, w, C);
+    uint32_t P = strip_width(h, w, C);
+    for (; strips && strips < 76 && P / 2 * C >= 32; strips *= 2) P /= 2;
+    return P;
+}
+
 cudaError_t permute_prepare() {
-    const void *fns[9] = {(const void *)strip_kernel<true>, (const void *)strip_kernel<false>,
+    const void *fns[11] = {(const void *)strip_kernel<true, 1024>, (const void *)strip_kernel<false, 1024>,
+                          (const void *)strip_kernel<true>, (const void *)strip_kernel<false>,
                           (const void *)strip_kernel<true, 256>, (const void *)strip_kernel<false, 256>,
                           (const void *)row_kernel<true>, (const void *)row_kernel<false>,
                           (const void *)row_kernel<true, 128>, (const void *)row_kernel<false, 128>,
@@ -447,8 +469,7 @@ cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
             tsm = tsm > g + 6ull * f.h ? tsm : g + 6ull * f.h;
             tab = tab && f.w / 4 <= 1024;
         }
-        constexpr size_t kSmPerSm = 233472, kReserved = 1024;
-        tab = tab && tsm <= kSmemLimit && kSmPerSm / (tsm + kReserved) >= kSmPerSm / (gsm + kReserved);
+        tab = tab && tsm <= kSmemLimit && kSmemPerSm / (tsm + kSmemReserved) >= kSmemPerSm / (gsm + kSmemReserved);
         if (gsm <= kSmemLimit) {
             gather_encrypt_kernel<<<b.perm_ctas, kGatherThreads, tab ? tsm : gsm, s>>>(b, 0, tab ? 1 : 0);
             note_launch();
@@ -461,34 +482,36 @@ cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
         if (b.f[k].N > b.f[big].N) big = k;
     uint32_t st, rt;
     cta_threads(b.f[big].h, b.f[big].w, b.f[big].C, &st, &rt);
-    auto rows = [&](bool enc) {
-        if (rt == 128) {
-            if (enc) row_kernel<true, 128><<<b.row_ctas, 128, rsm, s>>>(b, 0);
-            else row_kernel<false, 128><<<b.row_ctas, 128, rsm, s>>>(b, 0);
-        } else {
-            if (enc) row_kernel<true><<<b.row_ctas, kRowThreads, rsm, s>>>(b, 0);
-            else row_kernel<false><<<b.row_ctas, kRowThreads, rsm, s>>>(b, 0);
-        }
-        note_launch();
-        return cudaGetLastError();
+    // The second pass's launch overlaps the first's end: its CTAs wait in the kernel (2 us of a call).
+    auto launch = [&](auto *kernel, uint32_t grid, uint32_t threads, size_t smem, bool second) {
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = second ? 1 : 0;
+        const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, b, 0u);
+        if (err == cudaSuccess) note_launch();
+        return err != cudaSuccess ? err : cudaGetLastError();
     };
-    auto strips = [&](bool enc) {
-        if (st == 256) {
-            if (enc) strip_kernel<true, 256><<<b.perm_ctas, 256, ssm, s>>>(b, 0);
-            else strip_kernel<false, 256><<<b.perm_ctas, 256, ssm, s>>>(b, 0);
-        } else {
-            if (enc) strip_kernel<true><<<b.perm_ctas, kStripThreads, ssm, s>>>(b, 0);
-            else strip_kernel<false><<<b.perm_ctas, kStripThreads, ssm, s>>>(b, 0);
-        }
-        note_launch();
-        return cudaGetLastError();
+    auto rows = [&](bool second) {
+        if (rt == 128) return launch(encrypt ? row_kernel<true, 128> : row_kernel<false, 128>, b.row_ctas, 128, rsm, second);
+        return launch(encrypt ? row_kernel<true> : row_kernel<false>, b.row_ctas, kRowThreads, rsm, second);
     };
-    if (encrypt) {
-        if ((e = rows(true)) != cudaSuccess) return e;
-        return strips(true);
-    }
-    if ((e = strips(false)) != cudaSuccess) return e;
-    return rows(false);
+    auto strips = [&](bool second) {
+        if (st == 256)
+            return launch(encrypt ? strip_kernel<true, 256> : strip_kernel<false, 256>, b.perm_ctas, 256, ssm, second);
+        // one CTA to an SM by its shared memory: 1024 threads (a 1080p frame by itself, P = 64: encrypt 41 -> 37 us)
+        if (ssm > kSmemPerSm / 2 - kSmemReserved)
+            return launch(encrypt ? strip_kernel<true, 1024> : strip_kernel<false, 1024>, b.perm_ctas, 1024, ssm, second);
+        return launch(encrypt ? strip_kernel<true> : strip_kernel<false>, b.perm_ctas, kStripThreads, ssm, second);
+    };
+    if ((e = encrypt ? rows(false) : strips(false)) != cudaSuccess) return e;
+    return encrypt ? strips(true) : rows(true);
 }
 
 }  // namespace fhd

@@ -61,130 +61,152 @@ __device__ __forceinline__ void transpose4x4(uint32_t &a, uint32_t &b, uint32_t 
     d = __byte_perm(t1, t3, 0x7632);
 }
 
-// Column-word layout of a strip (the column pass's shared memory when h % 4 == 0).  A word holds four
-// consecutive rows of one byte column (row 4k + r in byte r).  The strip's QC byte columns form NL = QC / 4
-// column quads; the word of row quad p and column q = 4 lam + m sits at p * 4NL + m NL + lam.  A thread owns
-// one column quad lam and row quads p = p0, p0 + nq, ...: LT threads per row quad (NL, rounded up), so that the
-// threads of a warp take one or two row quads and the NL (or NL + 16) words they touch at a time lie in
-// distinct banks: with LT = 16 the pitch 4NL must be 16 mod 32.
-struct ColWords {
-    uint32_t NL, LT;
-};
-__device__ __forceinline__ ColWords col_words(uint32_t QC) {
-    const uint32_t NL = QC >> 2;
-    return {NL, NL <= 16 && (NL & 7) == 4 ? 16u : (NL + 31) & ~31u};
-}
-
-// Column pass over a strip in the column-word layout: for each column q of the strip, out[d][q] =
-// X[(d - s'_q) mod h][q] with s'_q = s_v (encrypt) or h - s_v (decrypt); X = G (encrypt) or E ^ B (decrypt),
-// and the output is XORed with B when encrypting.  With s'_q = 4 a + b:
+// Column pass over a strip in the column-word layout (shared memory when h % 4 == 0): for each column q of the
+// strip, out[d][q] = X[(d - s'_q) mod h][q] with s'_q = s_v (encrypt) or h - s_v (decrypt); X = G (encrypt) or
+// E ^ B (decrypt), and the output is XORed with B when encrypting.  A word holds four consecutive rows of one
+// byte column (row 4p + r in byte r); the strip's QC byte columns form NL = QC / 4 column quads, and the four
+// words of row quad p and column quad lam are the 16 bytes at p QC + 4 lam, column 4 lam + m in word m ^ x(lam).
+// A thread owns one column quad and kU row quads in turn.  With s'_q = 4 a + b:
 // * phase 1: the thread loads four rows of its four columns (one 32-bit word per row), transposes them into
 //   four column words and stores column q's word of row quad k at row quad (k + a) mod h/4: the rotation by
-//   whole row quads;
+//   whole row quads.  The swizzle x puts the words that the lanes store together into distinct banks, whatever
+//   their row quads, where QC is 0 or 16 mod 32;
 // * phase 2: output row quad t of column q is bytes 4 - b .. 7 - b of the column's words at row quads t - 1
-//   and t (one byte permute: the rest of the rotation), transposed back into four row words.
-// Every shared access is one 32-bit word per thread in distinct banks; every global access is a 32-bit word
-// per thread, consecutive across the threads of a row quad.
-template <bool kEnc, bool kL2, class Sync>
-__device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, ColWords cw, uint8_t *smem, uint32_t tid,
+//   and t (one byte permute: the rest of the rotation), both read by 16-byte loads, t - 1 from the turn before;
+//   transposed back into four row words by selectors that undo the swizzle.
+// Every global access is a 32-bit word per thread, consecutive across the threads of a row quad.
+//
+// Off: the type of offsets into the frame (32 bits below 4 GB).  What bounds the pass is latency, 96 bytes of a
+// row at a time: the strip fills the SM, so its two phases do not overlap.  The instructions were next, 218 a quad with
+// 64-bit offsets formed for each access and eight shared loads with their indices, and half that now.  A 4K frame
+// by itself, both passes: encrypt 51.4 -> 44.5 us, decrypt 53.8 -> 48.9 us, with CTAs of 1024 threads and the second
+// pass's launch beside the first (permute.cu).
+template <bool kEnc, bool kL2, class Off, class Sync>
+__device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uint8_t *smem, uint32_t tid,
                               uint32_t nthr, Sync sync) {
-    // row quads per thread and batch: 16 (8 in the persistent kernel, whose task bodies share 128 registers)
-    // independent 32-bit loads in flight
-    constexpr int kU = kL2 ? 2 : 4;
-    const uint32_t h = fd.h, w = fd.w, C = fd.C, H4 = h >> 2, NL = cw.NL, QP = QC;
-    const uint64_t rowB = (uint64_t)w * C, base = (uint64_t)j0 * C;
-    const uint64_t rw = rowB >> 2;   // 32-bit words per frame row
-    const uint8_t *src = kEnc ? fd.G : fd.src;
+    constexpr uint32_t kU = 2;   // row quads per thread and batch: 8 independent 32-bit loads in flight, B's one batch ahead
+    const uint32_t h = fd.h, w = fd.w, C = fd.C, H4 = h >> 2, NL = QC >> 2;
+    const Off row = (Off)w * C;
+    const uint8_t *src = kEnc ? fd.G : fd.src, *key = fd.B;
     uint8_t *out = kEnc ? fd.dst : fd.G;
     uint32_t *S = reinterpret_cast<uint32_t *>(smem);
-    [[maybe_unused]] const size_t words = (size_t)H4 * QP;
-    const uint32_t lam = tid % cw.LT, p0 = tid / cw.LT, nq = nthr / cw.LT;
-    const bool live = lam < NL;
-    // per column m of the thread's quad: whole row quads of the rotation (16 bits each) and the rest (2 bits)
-    uint32_t a01 = 0, a23 = 0, bs = 0;
-    const uint32_t *sp = reinterpret_cast<const uint32_t *>(src + base) + lam;
-    const uint32_t *bp = reinterpret_cast<const uint32_t *>(fd.B + base) + lam;
+    [[maybe_unused]] const size_t words = (size_t)H4 * QC;
+    // threads to a row quad: NL rounded up, so that a warp's row quads are whole (4 % faster than NL itself)
+    const uint32_t LT = NL <= 16 ? 16 : (NL + 31) & ~31u, lam = tid % LT, p0 = tid / LT, nq = nthr / LT;
+    const uint32_t x = (QC & 31 ? lam >> 2 : lam >> 3) & 3;
+    const bool live = lam < NL && p0 < nq;
+    const Off at0 = (Off)j0 * C + 4 * lam;   // this column quad in a row
+    // column m's rotation: whole row quads, and the byte selector of the rest
+    uint32_t a[4], sel[4];
+    auto load = [&](const uint8_t *p, Off at) -> uint32_t {
+        return FHD_IN(at + 3, fd.N, kSiteStripLoad) ? pass_ld<kL2>(reinterpret_cast<const uint32_t *>(p + at)) : 0;
+    };
     if (live) {
-        const FastMod modH(h);
+        const uint32_t M = 0xffffffffu / h + 1;   // v mod h = v - h floor(v M / 2^32) for v, h < 2^16, h >= 4
         const uint16_t *Dv = fd.D + (uint64_t)C * h;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             const uint32_t q = 4 * lam + m, jj = q / C, c = q - jj * C;
             const uint64_t dv = (uint64_t)c * w + j0 + jj;
-            const uint32_t t = FHD_IN(dv, (uint64_t)C * w, kSiteStripShift) ? modH.mod(pass_ld<kL2>(Dv + dv)) : 0;
-            const uint32_t sp2 = kEnc ? t : (t ? h - t : 0);
-            if (m < 2) a01 |= (sp2 >> 2) << (16 * m);
-            else a23 |= (sp2 >> 2) << (16 * (m - 2));
-            bs |= (sp2 & 3) << (2 * m);
+            const uint32_t v = FHD_IN(dv, (uint64_t)C * w, kSiteStripShift) ? pass_ld<kL2>(Dv + dv) : 0;
+            const uint32_t t = v - h * __umulhi(v, M);
+            const uint32_t sp = kEnc ? t : (t ? h - t : 0);
+            a[m] = sp >> 2;
+            sel[m] = 0x7654u - (sp & 3) * 0x1111u;
         }
-        for (uint32_t k0 = p0; k0 < H4; k0 += kU * nq) {
+        for (uint32_t k0 = p0 * kU; k0 < H4; k0 += nq * kU) {
             uint32_t v[kU][4];
+            Off at = at0 + (Off)(4 * k0) * row;
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const uint32_t k = k0 + u * nq;
+            for (uint32_t u = 0; u < kU; ++u)
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const uint64_t o = (uint64_t)(4 * k + r) * rw;
                     v[u][r] = 0;
-                    if (k < H4 && FHD_IN(base + 4 * (o + lam) + 3, fd.N, kSiteStripLoad)) {
-                        v[u][r] = pass_ld<kL2>(sp + o);
-                        if (!kEnc) v[u][r] ^= pass_ld<kL2>(bp + o);
+                    if (k0 + u < H4) {
+                        v[u][r] = load(src, at);
+                        if (!kEnc) v[u][r] ^= load(key, at);
                     }
+                    at += row;
                 }
+            uint32_t i[4];   // where column m's next word goes
+#pragma unroll
+            for (uint32_t m = 0; m < 4; ++m) {
+                const uint32_t p = k0 + a[m];
+                i[m] = (p >= H4 ? p - H4 : p) * QC + 4 * lam + (m ^ x);
             }
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const uint32_t k = k0 + u * nq;
-                if (k >= H4) break;
+            for (uint32_t u = 0; u < kU; ++u) {
+                if (k0 + u >= H4) break;
                 transpose4x4(v[u][0], v[u][1], v[u][2], v[u][3]);
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    uint32_t p = k + (((m < 2 ? a01 : a23) >> (16 * (m & 1))) & 0xffffu);
-                    p = p >= H4 ? p - H4 : p;
-                    const size_t i = (size_t)p * QP + m * NL + lam;
-                    if (FHD_IN(i, words, kSiteStripSmem)) S[i] = v[u][m];
+                    if (FHD_IN(i[m], words, kSiteStripSmem)) S[i[m]] = v[u][m];
+                    i[m] += QC;
+                    if (i[m] >= (uint32_t)words) i[m] -= (uint32_t)words;
                 }
             }
         }
     }
-    sync();
-    if (!live) return;
-    uint32_t *op = reinterpret_cast<uint32_t *>(out + base) + lam;
-    for (uint32_t t0 = p0; t0 < H4; t0 += kU * nq) {
-        uint32_t kb[kU][4];   // B words of the batch's output rows (encrypt), loaded before any store
-        if (kEnc) {
+    uint32_t kb[kU][4];   // B words of a batch's output rows (encrypt)
+    auto load_key = [&](uint32_t t0) {
+        Off at = at0 + (Off)(4 * t0) * row;
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const uint32_t t = t0 + u * nq;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint64_t o = (uint64_t)(4 * t + r) * rw;
-                    kb[u][r] = t < H4 && FHD_IN(base + 4 * (o + lam) + 3, fd.N, kSiteStripLoad) ? pass_ld<kL2>(bp + o) : 0;
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const uint32_t t = t0 + u * nq;
-            if (t >= H4) break;
-            const uint32_t tm = t ? t - 1 : H4 - 1;
-            uint32_t v[4];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const size_t i0 = (size_t)tm * QP + m * NL + lam, i1 = (size_t)t * QP + m * NL + lam;
-                const uint32_t sel = 0x7654u - ((bs >> (2 * m)) & 3) * 0x1111u;
-                v[m] = FHD_IN(i0, words, kSiteStripSmem) && FHD_IN(i1, words, kSiteStripSmem)
-                           ? __byte_perm(S[i0], S[i1], sel)
-                           : 0;
-            }
-            transpose4x4(v[0], v[1], v[2], v[3]);
+        for (uint32_t u = 0; u < kU; ++u)
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                const uint64_t o = (uint64_t)(4 * t + r) * rw;
-                if (!FHD_IN(base + 4 * (o + lam) + 3, fd.N, kSiteStripStore)) continue;
-                if (kEnc) __stcs(op + o, v[r] ^ kb[u][r]);
-                else op[o] = v[r];
+                kb[u][r] = t0 + u < H4 ? load(key, at) : 0;
+                at += row;
             }
+    };
+    if (kEnc && !kL2 && live) load_key(p0 * kU);
+    sync();
+    if (!live) return;
+    // selectors by place in the 16 bytes, and the transpose's, which put the columns back in order
+    uint32_t rot[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const uint32_t lo = x & 1 ? sel[m ^ 1] : sel[m], hi = x & 1 ? sel[m ^ 3] : sel[m ^ 2];
+        rot[m] = x & 2 ? hi : lo;
+    }
+    const uint32_t s0 = x & 1 ? 0x1504u : 0x5140u, s1 = x & 1 ? 0x3726u : 0x7362u;
+    const uint32_t s2 = x & 2 ? 0x1054u : 0x5410u, s3 = x & 2 ? 0x3276u : 0x7632u;
+    auto quad = [&](uint32_t p) -> uint4 {
+        const size_t i = (size_t)p * QC + 4 * lam;
+        return FHD_IN(i + 3, words, kSiteStripSmem) ? *reinterpret_cast<const uint4 *>(S + i) : make_uint4(0, 0, 0, 0);
+    };
+    for (uint32_t t0 = p0 * kU; t0 < H4; t0 += nq * kU) {
+        const Off first = at0 + (Off)(4 * t0) * row;
+        uint32_t kc[kU][4];
+        if (kEnc && kL2) load_key(t0);
+        if (kEnc) {
+#pragma unroll
+            for (uint32_t u = 0; u < kU; ++u)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) kc[u][r] = kb[u][r];
+        }
+        if (kEnc && !kL2) load_key(t0 + nq * kU);
+        uint4 before = quad(t0 ? t0 - 1 : H4 - 1);
+        Off at = first;
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u) {
+            if (t0 + u >= H4) break;
+            const uint4 now = quad(t0 + u);
+            const uint32_t v0 = __byte_perm(before.x, now.x, rot[0]), v1 = __byte_perm(before.y, now.y, rot[1]);
+            const uint32_t v2 = __byte_perm(before.z, now.z, rot[2]), v3 = __byte_perm(before.w, now.w, rot[3]);
+            const uint32_t y0 = __byte_perm(v0, v1, s0), y1 = __byte_perm(v0, v1, s1);
+            const uint32_t y2 = __byte_perm(v2, v3, s0), y3 = __byte_perm(v2, v3, s1);
+            const uint32_t o[4] = {__byte_perm(y0, y2, s2), __byte_perm(y0, y2, s3), __byte_perm(y1, y3, s2),
+                                   __byte_perm(y1, y3, s3)};
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                uint32_t *p = reinterpret_cast<uint32_t *>(out + at);
+                if (FHD_IN(at + 3, fd.N, kSiteStripStore)) {
+                    if (kEnc) __stcs(p, o[r] ^ kc[u][r]);
+                    else *p = o[r];
+                }
+                at += row;
+            }
+            before = now;
         }
     }
 }
@@ -209,12 +231,14 @@ __device__ void strip_pass(const FrameDesc &fd, uint32_t strip, uint8_t *smem, u
     uint8_t *S = smem;
     if (!FHD_IN(j0, w, kSiteStripSmem)) return;   // a strip past the frame (the same for the whole group)
     {
-        // the column-word route: rows of whole row quads, 32-bit aligned rows and pointers, and a strip whose
-        // column-word pitch is its row length (no padding: it fits the strip's shared memory)
-        const ColWords cw = col_words(QC);
-        if ((h & 3) == 0 && (QC & 3) == 0 && rowB % 4 == 0 && base % 4 == 0 && nthr % cw.LT == 0 &&
-            (cw.LT != 16 || (QC & 31) == 16) && aligned(src, 4) && aligned(out, 4) && aligned(fd.B, 4)) {
-            strip_pass_cw<kEnc, kL2>(fd, j0, QC, cw, smem, tid, nthr, sync);
+        // the column-word route: rows of whole row quads, 32-bit aligned rows and pointers (the strip's shared
+        // memory holds it without padding)
+        if ((h & 3) == 0 && (QC & 3) == 0 && rowB % 4 == 0 && base % 4 == 0 && nthr >= QC / 4 && aligned(src, 4) &&
+            aligned(out, 4) && aligned(fd.B, 4)) {
+            if (fd.N <= 0xffffffffu)
+                strip_pass_cw<kEnc, kL2, uint32_t>(fd, j0, QC, smem, tid, nthr, sync);
+            else
+                strip_pass_cw<kEnc, kL2, uint64_t>(fd, j0, QC, smem, tid, nthr, sync);
             return;
         }
     }
