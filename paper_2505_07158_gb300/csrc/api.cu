@@ -703,8 +703,9 @@ int persistent_side(fhd_cipher *c, uint32_t count, const fhd_frame *frames, bool
         d.T = p; p += align16(fhd::traj_bytes((uint64_t)d.C * (d.h + d.w), d.N, c->n));
         S.emits[k] = fhd::keystream_route() == FHD_KS_ROUTE_TRAJECTORY
                          ? (uint32_t)((d.N + fhd::kEmitTaskBytes - 1) / fhd::kEmitTaskBytes) : 0u;
-        // at most 64 pixels: the persistent column pass (352 threads) covers a strip row (<= 256 bytes) per pass
+        // the permutation group's threads cover a strip row (a thread a byte in the bytewise route)
         uint32_t P = std::min(fhd::strip_width(d.h, d.w, d.C), 64u);
+        while (P * d.C > fhd::persistent_mem_threads()) P /= 2;
         while (P > 1 && fhd::strip_smem_bytes(d.h, P, d.C) > lim) P /= 2;
         if (fhd::strip_smem_bytes(d.h, P, d.C) > lim)
             return fail(c, FHD_ERR_TOO_LARGE, "frame " + std::to_string(k) + ": too tall for a persistent launch");

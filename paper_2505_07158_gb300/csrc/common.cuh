@@ -142,6 +142,7 @@ struct PLaunch {
 
 cudaError_t launch_persistent(const PLaunch &L, size_t mem_smem, cudaStream_t s);
 size_t persistent_mem_smem_limit();   // shared memory the permutation tasks of a persistent launch may use
+uint32_t persistent_mem_threads();    // and the threads they run on
 
 // Chaining state of one video stream (Sec. II-A): x, y, z, w, gamma, frames done.
 struct StreamState {

@@ -4,7 +4,7 @@
 // lanes, and every rounded operation of the step waits for the one before: the step of chaos_dev.cuh is 27
 // such instructions and four exchanges, ~2.1k cycles, with the integer pipes idle.  The same roundings on
 // the integer pipes take ~20 cycles each.  Measured on GB300, the records of one 1080p frame (8,124 steps, one
-// warp): 5.22 ms, 1,330 cycles a step with the binary64 redoes below, against 8.53 ms.  What bounds it now is one
+// warp): 5.07 ms, 1,290 cycles a step with the binary64 redoes below, against 8.53 ms.  What bounds it now is one
 // warp's latency and issue together: a stage's chain is ~260 cycles (exchange 50, A B 50, T 30, k 30, c k 50, tin
 // 50) and its ~110 integer and ~40 float instructions take about as long to issue.
 //
@@ -233,9 +233,15 @@ __device__ __forceinline__ void int_stage(const IntVar &s, IntVar &t, const IntO
     const float T2f = __fmaf_rn(T1f, L.fM2, __fmul_rn(t.l.f, L.fo2));
     int_least(bad, l1, int_check(bad, T2f, L.d2));
     int_round(w0, w1, fbits(T2f) >> 23);
-    V = pack64(w0, w1) + q + T;
-    w0 = (uint32_t)V;
-    w1 = (uint32_t)(V >> 32);
+    {
+        uint32_t x0, x1;
+        asm("add.cc.u32 %0, %2, %4; addc.u32 %1, %3, %5;"
+            : "=&r"(x0), "=&r"(x1)
+            : "r"(w0), "r"(w1), "r"((uint32_t)q), "r"((uint32_t)(q >> 32)));
+        asm("add.cc.u32 %0, %2, %4; addc.u32 %1, %3, %5;"
+            : "=&r"(w0), "=&r"(w1)
+            : "r"(x0), "r"(x1), "r"((uint32_t)T), "r"((uint32_t)(T >> 32)));
+    }
     const float kf = __fadd_rn(T2f, qf), dk = __fadd_rn(L.dk, dq);
     int_least(bad, lq, int_check(bad, kf, dk));
     uint32_t up = 0, wk;

@@ -13,7 +13,7 @@
 //     is (Algorithm 1), then the frame's keystream tasks (Algorithm 2, the two sides interleaved): with the
 //     one-trajectory route one task per frame and side, the frame's trajectory records (traj_records in
 //     common.cuh); with the worker pairs one per three pairs;
-//   * warps 4 and 6-15: a permutation group of 352 threads with the CTA's large shared memory: per frame,
+//   * warps 4 and 6-11: a permutation group of 224 threads with the CTA's large shared memory: per frame,
 //     smallest first, the encryption's emission tasks (one-trajectory route: D and B from the records, in
 //     runs of kEmitTaskBytes of B), row bands and column strips, then the decryption's emission tasks,
 //     column strips and row bands (Sec. II-C, Algos 3-7, and the inverse).
@@ -38,15 +38,16 @@ namespace {
 // Warp roles by SM sub-partition (warp w runs on sub-partition w mod 4): the digest pipeline's consumers
 // (warps 0 and 1) and producer (warp 2, a chain worker afterwards) on sub-partitions 0, 1 and 2; the chain
 // workers (warps 2, 3 and 5) on sub-partitions 2, 3 and 1, one each -- in a digest CTA they start only after
-// its pipeline (below), so the digest rounds never share an issue port with a chain; warps 4 and 6-15 form
-// the permutation group.  Four warps per sub-partition leave each of them 128 registers (a
-// sub-partition's register file holds 16K).
-constexpr int kPWarps = 16;
+// its pipeline (below), so the digest rounds never share an issue port with a chain; warps 4 and 6-11 form
+// the permutation group.  Three warps per sub-partition leave each of them 168 registers (a sub-partition's
+// register file holds 16K): with four and 128 a chain's step took 15 % longer, a 4K frame's trajectory 24.2 ms
+// for 21.0, and the permutation group's four more warps gained back 0.3 ms at the end of a batch of 64.
+constexpr int kPWarps = 12;
 constexpr int kPThreads = 32 * kPWarps;
 constexpr int kChainWarps = 3;   // warps 2, 3, 5
 constexpr int kMemThreads = 32 * (kPWarps - 2 - kChainWarps);
 __device__ __forceinline__ int chain_index(uint32_t warp) { return warp == 2 ? 0 : warp == 3 ? 1 : warp == 5 ? 2 : -1; }
-__device__ __forceinline__ uint32_t mem_index(uint32_t warp) { return warp == 4 ? 0 : warp - 5; }   // warps 4, 6..15
+__device__ __forceinline__ uint32_t mem_index(uint32_t warp) { return warp == 4 ? 0 : warp - 5; }   // warps 4, 6..11
 constexpr unsigned kBarSha = 1, kBarMem = 2;
 // Shared memory: digests of the chain workers, broadcast slots and flag; then the digest pipeline's and, from
 // kPMemOffset, the permutation group's, which overlap: in a CTA with a pipeline the group starts after it.
@@ -382,8 +383,8 @@ __device__ bool wait_digest_cta(const PLaunch &L, volatile unsigned *flag) {
     return false;
 }
 
-// 16 warps x 128 registers fill the SM's register file: one CTA per SM, and no spills in the task bodies.
-__global__ void __maxnreg__(128) persistent_kernel(const __grid_constant__ PLaunch L) {
+// 12 warps x 168 registers fill the SM's register file: one CTA per SM, and no spills in the task bodies.
+__global__ void __maxnreg__(168) persistent_kernel(const __grid_constant__ PLaunch L) {
     extern __shared__ __align__(16) uint8_t smem[];
     uint8_t *H = smem;
     ShaSmem &sm = *reinterpret_cast<ShaSmem *>(smem + kPHeadSmem);
@@ -416,6 +417,7 @@ __global__ void __maxnreg__(128) persistent_kernel(const __grid_constant__ PLaun
 }  // namespace
 
 size_t persistent_mem_smem_limit() { return kPSmemLimit - kPMemOffset; }
+uint32_t persistent_mem_threads() { return kMemThreads; }
 
 cudaError_t launch_persistent(const PLaunch &L, size_t mem_smem, cudaStream_t s) {
     int dev = 0, sms = 0;

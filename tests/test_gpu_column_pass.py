@@ -45,3 +45,22 @@ def test_every_width(shape, P, threads):
     finally:
         fhd.fhd_set_strip_width(*shape, 0)
         fhd.fhd_set_cta_threads(*shape, 0, 0)
+
+
+@pytest.mark.parametrize("shape", [(60, 68, 4), (61, 67, 4), (64, 256, 4), (64, 256, 3), (33, 300, 1), (1028, 128, 4)])
+def test_strips_of_a_persistent_launch(shape):
+    """The widest strips for the permutation group's threads, word and byte routes, against the plain path."""
+    g = np.random.default_rng(7)
+    key = g.integers(0, 256, size=32, dtype=np.uint8).tobytes()
+    F = torch.from_numpy(g.integers(0, 256, size=shape, dtype=np.uint8)).cuda()
+    out = []
+    for persistent in (False, True):
+        c = fhd.Cipher(key)
+        s, E, H = c.open_stream(key), torch.empty_like(F), torch.zeros(32, dtype=torch.uint8, device="cuda")
+        (c.encrypt_frames_persistent if persistent else c.encrypt_frames)([(s, F, E, H)])
+        d = fhd.Cipher(key)
+        P = torch.empty_like(F)
+        (d.decrypt_frames_persistent if persistent else d.decrypt_frames)([(d.open_stream(key), E, P, H)])
+        assert torch.equal(P, F)
+        out.append(E)
+    assert torch.equal(out[0], out[1])
