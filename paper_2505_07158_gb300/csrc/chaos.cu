@@ -192,7 +192,8 @@ IntStepTab int_step_tab(double h) {
             const double k = t2[v] + q[v] + u * kmax[v];
             d1[v] = std::max(d1[v], t1[v]);
             d2[v] = std::max(d2[v], t2[v]);
-            dk[v] = std::max(dk[v], t2[v] + 3 * u * kmax[v]);
+            // k's own rounding, a sixth of those of acc (14 u) and of c acc (12 u) and what is left of c k's
+            dk[v] = std::max(dk[v], t2[v] + 5 * u * kmax[v] + 2 * u * kmax[v] / 6);
             amax[v] += f * kmax[v];
             acc[v] += f * k + u * amax[v];
             e[v] = es[v] + c * (st == 3 ? acc[v] : k) + 2 * u * c * (st == 3 ? amax[v] : kmax[v]) + u * lim[v];
@@ -202,11 +203,11 @@ IntStepTab int_step_tab(double h) {
     const int grid_kappa[4] = {int_kappa(0), int_kappa(1), int_kappa(2), int_kappa(3)};
     const int sA[4] = {-1, 0, 0, 1}, sB[4] = {3, 2, 1, 2};
     for (int v = 0; v < 4; ++v) {
-        const double scale = 1.1 * std::ldexp(1.0, grid_kappa[v]);
+        const double scale = 1.25 * std::ldexp(1.0, grid_kappa[v]);   // and the roundings of the bounds and checks
         t.d1[v] = (float)(scale * d1[v]);
         t.d2[v] = (float)(scale * d2[v]);
         t.dk[v] = (float)(scale * dk[v]);
-        t.dt[v] = (float)(scale * (es[v] + u * lim[v] + 2 * u * h * kmax[v]));
+        t.dt[v] = (float)(scale * (es[v] + 2 * u * lim[v] + 2 * u * h * kmax[v]));
         t.limit[v] = (float)std::ldexp(lim[v], grid_kappa[v]);
         // |A~| qA + |B~| qB in this lane's scale: A~, B~ carry their own lanes' scales
         const double eA = sA[v] < 0 ? 0x1p-22 : et[sA[v]], eB = et[sB[v]], lB = lim[sB[v]], lA = sA[v] < 0 ? 1.0 : lim[sA[v]];

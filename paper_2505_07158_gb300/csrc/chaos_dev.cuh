@@ -254,7 +254,7 @@ struct Chains {
         load(binary64_redo(s, lane, gamma, c.h, c.hh, c.h6), lane);
     }
     // `count` steps, each after before_step(m48, i), i its number.  The loop without the redo's call in it keeps its
-    // registers in place: 5.07 ms for the records of a 1080p frame, 5.34 ms with a call of step() per turn.
+    // registers in place: 5.07 ms for the records of a 1080p frame, where it took 5.34 ms with a call of step() per turn.
     template <class F>
     __device__ __forceinline__ void steps(uint64_t count, int lane, F &&before_step) {
         for (uint64_t i = 0; i < count;) {

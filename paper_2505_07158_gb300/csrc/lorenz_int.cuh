@@ -4,7 +4,7 @@
 // lanes, and every rounded operation of the step waits for the one before: the step of chaos_dev.cuh is 27
 // such instructions and four exchanges, ~2.1k cycles, with the integer pipes idle.  The same roundings on
 // the integer pipes take ~20 cycles each.  Measured on GB300, the records of one 1080p frame (8,124 steps, one
-// warp): 5.07 ms, 1,290 cycles a step with the binary64 redoes below, against 8.53 ms.  What bounds it now is one
+// warp): 5.11 ms, 1,300 cycles a step with the binary64 redoes below, against 8.53 ms.  What bounds it now is one
 // warp's latency and issue together: a stage's chain is ~260 cycles (exchange 50, A B 50, T 30, k 30, c k 50, tin
 // 50) and its ~110 integer and ~40 float instructions take about as long to issue.
 //
@@ -27,7 +27,7 @@
 // stages for |x| < 28, |y| < 30, |z| < 50, |w| < 216); a shadow within its bound of a power of two or of the
 // smallest magnitude its grid carries, a variable outside those ranges, and a factor whose low bits are all
 // zero (only then could a product be a tie: 51 zero bits in both factors together) mark the step, and a marked step
-// is done again in binary64.  On the attractor that is about 1.7 % of the steps at h = 0.01 (2.3 % with ranges of
+// is done again in binary64.  On the attractor that is about 2 % of the steps at h = 0.01 (2.6 % with ranges of
 // 32, 32, 64, 256 and grids of 62 and 60).  Three constants of the step (h/2, h, h/6) and gamma
 // have to be in range for the shifts (IntStepTab::ok, int_gamma_ok); otherwise every step is binary64.
 #pragma once
