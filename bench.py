@@ -250,7 +250,7 @@ def traj_steps(h, w, C, n):
     return R + 2 - 2 * n
 
 
-RK4_FP64_INSTR = 27     # binary64 instructions one warp issues per RK4 step of its chains (six-chain layout)
+RK4_CHAIN_CYCLES = 1040  # dependency chain of one RK4 step on the integer pipes: four stages of ~260 cycles
 
 
 def sha_blocks(N, n):
@@ -753,30 +753,29 @@ def run_ours(args):
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
 
     def traj_roof(k):
-        # One chain per frame, strictly sequential: the launch lasts its longest chain, whose warp issues 27
-        # binary64 instructions per step back to back on one sub-partition's binary64 pipe.  achieved = the
-        # binary64 lane-operations that warp issues per second (steps x 27 x 32 / launch time alone), peak =
-        # one sub-partition's share of the measured binary64 peak: frac is how close the chain runs to the
-        # pipe's own rate.  The whole GPU's binary64 fraction (algorithmic ops of all launches over the union
-        # of their spans) is reported beside it.
+        # One chain per frame, strictly sequential: the launch lasts its longest chain, one warp's RK4 steps on
+        # the integer pipes.  achieved = its steps per second (launch time alone), peak = the steps per second of
+        # the step's dependency chain at the sampled clock: frac is how much of the launch that chain takes (the
+        # rest is the warp's issue and the steps done again in binary64).  The whole GPU's binary64 fraction
+        # (algorithmic ops of all launches over the union of their spans) is reported beside it.
         steps = traj_steps(HGT, WID, CH, N_WORKERS)
         ms = alone[k][0] / alone[k][1]
-        sp_peak = fp64_peak * 1e12 / (sms * 4) / 1e9
-        ach = steps * RK4_FP64_INSTR * 32 / (ms / 1000.0) / 1e9
+        mhz = clocks_mhz or 2070.0
+        ach, peak = steps / (ms / 1000.0), mhz * 1e6 / RK4_CHAIN_CYCLES
         n_l = kern[k]["launches_per_step"] * args.steps
         gpu_ach = n_l * steps * per_step_frames * RK4_FP64_OPS / (busy_ms(k) / 1000.0) / 1e12
-        return {"bound": "alu", "achieved": ach, "peak": sp_peak, "unit": "Gop/s (binary64 lane-ops, one sub-partition)",
-                "frac": ach / sp_peak, "traffic": TRAFFIC_TRAJ_PER_FRAME * per_step_frames,
-                "peak_source": fp64_source + f", divided by {sms} SMs x 4 sub-partitions",
-                "per_launch_units": f"{per_step_frames} frames x one trajectory of {steps} RK4 steps "
-                                    f"({RK4_FP64_INSTR} binary64 warp instructions each) + the D/B emission",
+        return {"bound": "latency", "achieved": ach, "peak": peak, "unit": "RK4 steps/s of one chain",
+                "frac": ach / peak, "traffic": TRAFFIC_TRAJ_PER_FRAME * per_step_frames,
+                "peak_source": f"{RK4_CHAIN_CYCLES} cycles of dependent instructions per step at {mhz:.0f} MHz",
+                "per_launch_units": f"{per_step_frames} frames x one trajectory of {steps} RK4 steps + the D/B emission",
                 "timing": "one launch (trajectory + emission) with nothing else running",
                 "ms_per_launch_alone": ms, "ms_per_launch_in_timed_run": kern[k]["avg_launch_ms"],
                 "step_cycles_alone": (ms / 1000.0) * (clocks_mhz or 0) * 1e6 / steps if clocks_mhz else None,
                 "gpu_binary64_frac": gpu_ach / fp64_peak,
                 "gpu_binary64_note": f"{steps} steps x {RK4_FP64_OPS} ops per frame, all launches over the union "
-                                     "of their spans, against the whole GPU's measured peak: the route needs "
-                                     "one chain per frame, so the pipes stay mostly idle"}
+                                     "of their spans, against the whole GPU's measured peak: the route needs one "
+                                     "chain per frame and takes it on the integer pipes, so the binary64 pipes stay "
+                                     "mostly idle"}
 
     roofs = {}
     clocks_mhz = clk.summary().get("sm_mhz")
