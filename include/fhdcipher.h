@@ -367,7 +367,9 @@ int fhd_permute_decrypt(const uint8_t *src, uint8_t *dst, uint32_t height, uint3
                         uint32_t channels, const uint16_t *D, const uint8_t *B, void *stream);
 
 /* Strip width (pixels) the permutation kernels use for this shape, and the
- * override hook of the autotuner: 0 restores the built-in choice. */
+ * override hook of the autotuner: 0 restores the built-in choice.  A launch
+ * whose strips at the built-in widths would leave more than half of the SMs
+ * idle takes narrower ones. */
 uint32_t fhd_strip_width(uint32_t height, uint32_t width, uint32_t channels);
 int fhd_set_strip_width(uint32_t height, uint32_t width, uint32_t channels, uint32_t P);
 
@@ -379,8 +381,8 @@ int fhd_set_row_band(uint32_t height, uint32_t width, uint32_t channels, uint32_
 
 
 /* Threads per CTA of the permutation passes for frames of one shape (autotuner
- * hook): the column pass 256 or 512 (default 512, two CTAs per SM; 256 runs four
- * per SM), the row pass 128 or 256 (default 256, six CTAs per SM; 128 runs
+ * hook): the column pass 256 or 512 (default 512, two CTAs per SM, and 1024
+ * threads where the strips leave room for one; 256 runs four per SM), the row pass 128 or 256 (default 256, six CTAs per SM; 128 runs
  * twelve); 0 keeps the default.  A batch takes the choice of its largest frame's
  * shape.  Results are the same for every value.  FHD_ERR_INVALID_ARG for another
  * value or a bad shape, FHD_ERR_TOO_LARGE when the override table (64 shapes) is

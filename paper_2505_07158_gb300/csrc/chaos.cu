@@ -37,7 +37,7 @@
 // finite (an overflowing 2 k makes the definition's state non-finite anyway).
 //
 // LHCS_m, the trajectory kernel and the one-pair worker kernel step on the integer pipes instead (Chains in
-// chaos_dev.cuh, lorenz_int.cuh): ~1.6k cycles a step, bit-identical.  That costs issue slots, which a warp that
+// chaos_dev.cuh, lorenz_int.cuh): ~1.3k cycles a step, bit-identical.  That costs issue slots, which a warp that
 // has its sub-partition to itself does not miss; the worker-pair launches that fill the GPU with chains keep the
 // binary64 steps above, six or eight chains to a warp.
 #include <algorithm>
@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(256) keystream_kernel(const __grid_constant__ 
 // Warps per CTA of the kernels whose chains step on the integer pipes: one to each of the SM's sub-partitions.
 // With one-warp CTAs two chains may meet on a sub-partition while others are free, which costs a pipeline of many
 // launches: the clip pipeline (720 trajectories in flight) 11.3k frames/s, 13.1k with four warps per CTA, and a
-// single launch the same either way (6.29 ms for 30 frames).  Two frames to a warp, 6.55 ms and 13.8k, were left:
-// marked steps of either frame hold both up.
+// single launch the same either way (measured with a step of 1,580 cycles; 13.9k with the present one).  Two frames
+// to a warp, 4 % slower by themselves, were left: marked steps of either frame hold both up.
 constexpr uint32_t kIntWarps = 4;
 
 // One worker pair per one-warp CTA, its two chains on the integer pipes (lorenz_int.cuh).

@@ -216,7 +216,7 @@ __device__ __noinline__ void mem_task(uint32_t kind, const FrameDesc &fd, uint32
     else emit_task(fd, n, idx, mtid);
 }
 
-// ---- chain workers (warps 2-5): LHCS_m tasks, then worker warps
+// ---- chain workers (warps 2, 3 and 5): LHCS_m tasks, then worker warps
 __device__ void chain_worker(const PLaunch &L, uint8_t *H) {
     const int lane = threadIdx.x & 31;
     // One lane waits; the warp learns the outcome.
