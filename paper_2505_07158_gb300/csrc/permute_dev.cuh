@@ -289,33 +289,36 @@ __device__ void strip_pass(const FrameDesc &fd, uint32_t strip, uint8_t *smem, u
             }
         }
     } else {
-        const uint32_t RT = nthr / QC;
-        if (tid < QC * RT) {
-            const uint32_t q = tid % QC, tr = tid / QC;
-            const uint32_t jj = q / C, c = q - jj * C;
-            const uint64_t dv = (uint64_t)c * w + j0 + jj;
-            const uint32_t t = FHD_IN(dv, (uint64_t)C * w, kSiteStripShift) ? modH.mod(pass_ld<kL2>(Dv + dv)) : 0;
-            const uint32_t ht = kEnc ? t : h - t;
-            for (uint32_t i = tr; i < h; i += RT) {
-                const uint64_t o = (uint64_t)i * rowB + base + q;
-                uint8_t e = 0;
-                if (FHD_IN(o, fd.N, kSiteStripLoad)) {
-                    e = pass_ld<kL2>(src + o);
-                    if (!kEnc) e ^= pass_ld<kL2>(fd.B + o);
+        // a thread per byte of a strip row; where the row has more bytes than the group threads, several in turn
+        const uint32_t nq = min(QC, nthr), RT = nthr / nq;
+        if (tid < nq * RT) {
+            const uint32_t tr = tid / nq;
+            for (uint32_t q = tid % nq; q < QC; q += nq) {
+                const uint32_t jj = q / C, c = q - jj * C;
+                const uint64_t dv = (uint64_t)c * w + j0 + jj;
+                const uint32_t t = FHD_IN(dv, (uint64_t)C * w, kSiteStripShift) ? modH.mod(pass_ld<kL2>(Dv + dv)) : 0;
+                const uint32_t ht = kEnc ? t : h - t;
+                for (uint32_t i = tr; i < h; i += RT) {
+                    const uint64_t o = (uint64_t)i * rowB + base + q;
+                    uint8_t e = 0;
+                    if (FHD_IN(o, fd.N, kSiteStripLoad)) {
+                        e = pass_ld<kL2>(src + o);
+                        if (!kEnc) e ^= pass_ld<kL2>(fd.B + o);
+                    }
+                    uint32_t d = i + ht;
+                    d = d >= h ? d - h : d;
+                    if (FHD_IN((size_t)d * RP + q, (size_t)h * RP, kSiteStripSmem)) S[(size_t)d * RP + q] = e;
                 }
-                uint32_t d = i + ht;
-                d = d >= h ? d - h : d;
-                if (FHD_IN((size_t)d * RP + q, (size_t)h * RP, kSiteStripSmem)) S[(size_t)d * RP + q] = e;
             }
         }
     }
     sync();
 
     // ---- phase 2: the strip leaves row by row (XORed with B when encrypting)
-    const uint32_t nv = QC / vec;
-    const uint32_t RT = nthr / nv;
-    if (tid >= nv * RT) return;
-    const uint32_t tv = tid % nv, tr = tid / nv;
+    const uint32_t nv = QC / vec, nt = min(nv, nthr);
+    const uint32_t RT = nthr / nt;
+    if (tid >= nt * RT) return;
+    const uint32_t tv = tid % nt, tr = tid / nt;
     if (vec == 16) {
         for (uint32_t ib = tr; ib < h; ib += kRowsV * RT) {
             uint4 g[kRowsV], k4[kRowsV];
@@ -349,12 +352,14 @@ __device__ void strip_pass(const FrameDesc &fd, uint32_t strip, uint8_t *smem, u
             *reinterpret_cast<uint32_t *>(out + o) = g;
         }
     } else {
-        for (uint32_t i = tr; i < h; i += RT) {
-            const uint64_t o = (uint64_t)i * rowB + base + tv;
-            if (!FHD_IN((size_t)i * RP + tv, (size_t)h * RP, kSiteStripSmem) || !FHD_IN(o, fd.N, kSiteStripStore)) continue;
-            uint8_t g = S[(size_t)i * RP + tv];
-            if (kEnc) g ^= pass_ld<kL2>(fd.B + o);
-            out[o] = g;
+        for (uint32_t q = tv; q < QC; q += nt) {
+            for (uint32_t i = tr; i < h; i += RT) {
+                const uint64_t o = (uint64_t)i * rowB + base + q;
+                if (!FHD_IN((size_t)i * RP + q, (size_t)h * RP, kSiteStripSmem) || !FHD_IN(o, fd.N, kSiteStripStore)) continue;
+                uint8_t g = S[(size_t)i * RP + q];
+                if (kEnc) g ^= pass_ld<kL2>(fd.B + o);
+                out[o] = g;
+            }
         }
     }
 }
