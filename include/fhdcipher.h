@@ -381,12 +381,13 @@ int fhd_set_row_band(uint32_t height, uint32_t width, uint32_t channels, uint32_
 
 
 /* Threads per CTA of the permutation passes for frames of one shape (autotuner
- * hook): the column pass 256 or 512 (default 512, two CTAs per SM, and 1024
- * threads where the strips leave room for one; 256 runs four per SM), the row pass 128 or 256 (default 256, six CTAs per SM; 128 runs
- * twelve); 0 keeps the default.  A batch takes the choice of its largest frame's
+ * hook): the column pass 256 (four CTAs per SM) or 512 (two), the row pass 128
+ * (twelve) or 256 (six).  0 leaves the choice to the launch: 256 for the row
+ * pass; for the column pass 512, and 1024 where the strips' shared memory leaves
+ * room for one CTA to an SM.  A batch takes the choice of its largest frame's
  * shape.  Results are the same for every value.  FHD_ERR_INVALID_ARG for another
  * value or a bad shape, FHD_ERR_TOO_LARGE when the override table (64 shapes) is
- * full.  fhd_cta_threads reports the choice in effect. */
+ * full.  fhd_cta_threads reports the values set, and 512 and 256 where none is. */
 int fhd_set_cta_threads(uint32_t height, uint32_t width, uint32_t channels, uint32_t strip_threads,
                         uint32_t row_threads);
 int fhd_cta_threads(uint32_t height, uint32_t width, uint32_t channels, uint32_t *strip_threads,

@@ -674,12 +674,13 @@ def fhd_set_row_band(height: int, width: int, channels: int, RB: int):
 
 def fhd_set_cta_threads(height: int, width: int, channels: int, strip_threads: int = 0, row_threads: int = 0):
     """Threads per CTA of the permutation passes for one frame shape (column pass 256/512, row pass 128/256;
-    0 keeps the default)."""
+    0 leaves the choice to the launch)."""
     _check(load().fhd_set_cta_threads(height, width, channels, strip_threads, row_threads))
 
 
 def fhd_cta_threads(height: int, width: int, channels: int) -> tuple:
-    """(column-pass, row-pass) threads per CTA in effect for a frame shape."""
+    """(column-pass, row-pass) threads per CTA set for a frame shape; 512 and 256 where none are (the column pass of
+    such a shape takes 1024 where its strips leave room for one CTA to an SM)."""
     a, b = ctypes.c_uint32(), ctypes.c_uint32()
     _check(load().fhd_cta_threads(height, width, channels, ctypes.byref(a), ctypes.byref(b)))
     return int(a.value), int(b.value)

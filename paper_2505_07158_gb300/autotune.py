@@ -6,8 +6,8 @@ Per frame shape (height, width, channels) it chooses, by timing:
   memory.  Wide strips amortise the per-row work; narrow ones let two or more CTAs share an SM and hide
   memory latency.  Every power-of-two P whose strip fits is timed.
 * RB, the rows per CTA of the row pass (bands of whole rows staged in shared memory), at the chosen P.
-* ST and RT, the threads per CTA of the column pass (256 or 512) and of the row pass (128 or 256), at the
-  chosen P and RB.
+* ST and RT, the threads per CTA of the column pass (256, 512 or the launch's own choice, 0) and of the row pass
+  (128 or 256), at the chosen P and RB.
 
 Each candidate is timed as the batched encrypt + decrypt permutation launches per frame of a batch of up to
 30 frames (CUDA events the library records on the launch stream, median of several runs); the fastest is
@@ -134,7 +134,7 @@ def batch_frames(h: int, w: int, C: int) -> int:
     return max(4, min(30, int(1.5e9 // (h * w * C))))
 
 
-CTA_CANDIDATES = ((512, 256), (256, 256), (512, 128))
+CTA_CANDIDATES = ((0, 256), (512, 256), (256, 256), (0, 128))
 
 
 def tune_shape(h: int, w: int, C: int, reps: int = 7) -> dict:

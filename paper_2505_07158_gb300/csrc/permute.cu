@@ -320,7 +320,7 @@ uint32_t permute_strips(uint32_t w, uint32_t P) { return (w + P - 1) / P; }
 static uint32_t g_override_key[64][3];
 static uint32_t g_override_P[64];
 static uint32_t g_override_RB[64];
-static uint32_t g_override_ST[64];   // column-pass threads per CTA (0: kStripThreads)
+static uint32_t g_override_ST[64];   // column-pass threads per CTA (0: the launch's choice, strip_threads)
 static uint32_t g_override_RT[64];   // row-pass threads per CTA (0: kRowThreads)
 static int g_overrides = 0;
 
@@ -352,6 +352,16 @@ void cta_threads(uint32_t h, uint32_t w, uint32_t C, uint32_t *st, uint32_t *rt)
             if (g_override_ST[k]) *st = g_override_ST[k];
             if (g_override_RT[k]) *rt = g_override_RT[k];
         }
+}
+
+// Threads of a column pass with smem bytes of shared memory to a CTA, for a batch whose largest frame has this shape: the
+// override's, or 512, two CTAs to an SM, and 1024 where there is room for one CTA (a 1080p frame by itself, P = 64:
+// encrypt 41 -> 37 us).
+static uint32_t strip_threads(uint32_t h, uint32_t w, uint32_t C, size_t smem) {
+    for (int k = 0; k < g_overrides; ++k)
+        if (g_override_key[k][0] == h && g_override_key[k][1] == w && g_override_key[k][2] == C && g_override_ST[k])
+            return g_override_ST[k];
+    return smem > kSmemPerSm / 2 - kSmemReserved ? 1024 : kStripThreads;
 }
 
 int set_strip_override(uint32_t h, uint32_t w, uint32_t C, uint32_t P) {
@@ -482,6 +492,7 @@ cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
         if (b.f[k].N > b.f[big].N) big = k;
     uint32_t st, rt;
     cta_threads(b.f[big].h, b.f[big].w, b.f[big].C, &st, &rt);
+    st = strip_threads(b.f[big].h, b.f[big].w, b.f[big].C, ssm);
     // The second pass's launch overlaps the first's end: its CTAs wait in the kernel (2 us of a call).
     auto launch = [&](auto *kernel, uint32_t grid, uint32_t threads, size_t smem, bool second) {
         cudaLaunchAttribute at[1];
@@ -505,8 +516,7 @@ cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
     auto strips = [&](bool second) {
         if (st == 256)
             return launch(encrypt ? strip_kernel<true, 256> : strip_kernel<false, 256>, b.perm_ctas, 256, ssm, second);
-        // one CTA to an SM by its shared memory: 1024 threads (a 1080p frame by itself, P = 64: encrypt 41 -> 37 us)
-        if (ssm > kSmemPerSm / 2 - kSmemReserved)
+        if (st == 1024)
             return launch(encrypt ? strip_kernel<true, 1024> : strip_kernel<false, 1024>, b.perm_ctas, 1024, ssm, second);
         return launch(encrypt ? strip_kernel<true> : strip_kernel<false>, b.perm_ctas, kStripThreads, ssm, second);
     };
