@@ -52,16 +52,12 @@ __device__ __forceinline__ uint32_t find_frame(const Batch &b, uint32_t cta) {
     return lo;
 }
 
-// The second pass of a call is launched while the first still runs (launch_second) and waits here for its end.
-__device__ __forceinline__ void wait_for_first_pass() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 template <bool kEnc, int kT = kStripThreads>
 __global__ void __launch_bounds__(kT, strip_ctas_per_sm<kT>()) strip_kernel(const __grid_constant__ Batch b,
                                                                             uint32_t cta_base) {
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<false>(b, cta)];
-    wait_for_first_pass();
     strip_pass<kEnc>(fd, cta - fd.cta0, smem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
@@ -71,7 +67,6 @@ __global__ void __launch_bounds__(kT, row_ctas_per_sm<kT>()) row_kernel(const __
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<true>(b, cta)];
-    wait_for_first_pass();
     row_pass<kEnc>(fd, cta - fd.rcta0, smem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
@@ -251,7 +246,6 @@ __global__ void __launch_bounds__(kGatherThreads, 2) gather_encrypt_kernel(const
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<false>(b, cta)];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t h = fd.h, w = fd.w, P = fd.P;
     const uint32_t j0 = (cta - fd.cta0) * P;
     if (!FHD_IN(j0, w, kSiteGatherSmem)) return;   // a strip past the frame (the whole CTA)
@@ -493,35 +487,36 @@ cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
     uint32_t st, rt;
     cta_threads(b.f[big].h, b.f[big].w, b.f[big].C, &st, &rt);
     st = strip_threads(b.f[big].h, b.f[big].w, b.f[big].C, ssm);
-    // The second pass's launch overlaps the first's end: its CTAs wait in the kernel (2 us of a call).
-    auto launch = [&](auto *kernel, uint32_t grid, uint32_t threads, size_t smem, bool second) {
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cfg.attrs = at;
-        cfg.numAttrs = second ? 1 : 0;
-        const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, b, 0u);
-        if (err == cudaSuccess) note_launch();
-        return err != cudaSuccess ? err : cudaGetLastError();
+    // (Launching the second pass with programmatic stream serialization, so that its launch overlaps the first's end,
+    // saved 2 us of a call by itself.  It is not done: with more calls in flight than hardware queues, the pass that
+    // waits holds up the queue it shares, 12 calls of 8 720p frames on 8 queues 12.5 ms against 7.3.)
+    auto rows = [&] {
+        if (rt == 128) {
+            if (encrypt) row_kernel<true, 128><<<b.row_ctas, 128, rsm, s>>>(b, 0);
+            else row_kernel<false, 128><<<b.row_ctas, 128, rsm, s>>>(b, 0);
+        } else {
+            if (encrypt) row_kernel<true><<<b.row_ctas, kRowThreads, rsm, s>>>(b, 0);
+            else row_kernel<false><<<b.row_ctas, kRowThreads, rsm, s>>>(b, 0);
+        }
+        note_launch();
+        return cudaGetLastError();
     };
-    auto rows = [&](bool second) {
-        if (rt == 128) return launch(encrypt ? row_kernel<true, 128> : row_kernel<false, 128>, b.row_ctas, 128, rsm, second);
-        return launch(encrypt ? row_kernel<true> : row_kernel<false>, b.row_ctas, kRowThreads, rsm, second);
+    auto strips = [&] {
+        if (st == 256) {
+            if (encrypt) strip_kernel<true, 256><<<b.perm_ctas, 256, ssm, s>>>(b, 0);
+            else strip_kernel<false, 256><<<b.perm_ctas, 256, ssm, s>>>(b, 0);
+        } else if (st == 1024) {
+            if (encrypt) strip_kernel<true, 1024><<<b.perm_ctas, 1024, ssm, s>>>(b, 0);
+            else strip_kernel<false, 1024><<<b.perm_ctas, 1024, ssm, s>>>(b, 0);
+        } else {
+            if (encrypt) strip_kernel<true><<<b.perm_ctas, kStripThreads, ssm, s>>>(b, 0);
+            else strip_kernel<false><<<b.perm_ctas, kStripThreads, ssm, s>>>(b, 0);
+        }
+        note_launch();
+        return cudaGetLastError();
     };
-    auto strips = [&](bool second) {
-        if (st == 256)
-            return launch(encrypt ? strip_kernel<true, 256> : strip_kernel<false, 256>, b.perm_ctas, 256, ssm, second);
-        if (st == 1024)
-            return launch(encrypt ? strip_kernel<true, 1024> : strip_kernel<false, 1024>, b.perm_ctas, 1024, ssm, second);
-        return launch(encrypt ? strip_kernel<true> : strip_kernel<false>, b.perm_ctas, kStripThreads, ssm, second);
-    };
-    if ((e = encrypt ? rows(false) : strips(false)) != cudaSuccess) return e;
-    return encrypt ? strips(true) : rows(true);
+    if ((e = encrypt ? rows() : strips()) != cudaSuccess) return e;
+    return encrypt ? strips() : rows();
 }
 
 }  // namespace fhd

@@ -79,8 +79,7 @@ __device__ __forceinline__ void transpose4x4(uint32_t &a, uint32_t &b, uint32_t 
 // Off: the type of offsets into the frame (32 bits below 4 GB).  What bounds the pass is latency, 96 bytes of a
 // row at a time: the strip fills the SM, so its two phases do not overlap.  The instructions were next, 218 a quad with
 // 64-bit offsets formed for each access and eight shared loads with their indices, and half that now.  A 4K frame
-// by itself, both passes: encrypt 51.4 -> 44.5 us, decrypt 53.8 -> 48.9 us, with CTAs of 1024 threads and the second
-// pass's launch beside the first (permute.cu).
+// by itself, both passes: encrypt 51.4 -> 44.5 us, decrypt 53.8 -> 48.9 us, with CTAs of 1024 threads.
 template <bool kEnc, bool kL2, class Off, class Sync>
 __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uint8_t *smem, uint32_t tid,
                               uint32_t nthr, Sync sync) {
