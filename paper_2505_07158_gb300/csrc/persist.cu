@@ -110,7 +110,7 @@ __device__ __forceinline__ uint32_t segment(const uint32_t *a, uint32_t m, uint3
 __device__ __forceinline__ void digest_task(const PLaunch &L, uint32_t task, uint32_t rtid, ShaSmem &sm) {
     const PSide &S = L.s[0];
     const uint32_t n = S.n;
-    sha_pipeline<true>(
+    sha_pipeline<false>(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             if (!FHD_IN(m / n, S.count, kSiteShaDigest) || !FHD_IN(L.prio[m / n], S.count, kSitePersistTask))
                 return false;
@@ -134,13 +134,13 @@ __device__ void digest_worker(const PLaunch &L, ShaSmem &sm, unsigned *slot) {
     const uint32_t n = S.n, nmsg = S.count * n;
     for (;;) {
         if (rtid == 0) slot[0] = ld_acquire(&L.cnt->abort) ? L.sha_units : atomicAdd(&L.cnt->sha_next, 1u);
-        bar_sync(kBarSha, kShaThreads<true>);
+        bar_sync(kBarSha, kShaThreads);
         const uint32_t task = slot[0];
-        bar_sync(kBarSha, kShaThreads<true>);
+        bar_sync(kBarSha, kShaThreads);
         if (task >= L.sha_units) return;
         digest_task(L, task, rtid, sm);
         __threadfence();
-        bar_sync(kBarSha, kShaThreads<true>);
+        bar_sync(kBarSha, kShaThreads);
         if (rtid == 0) {
             // the frames this task's messages belong to: count them in, and the task that completes a
             // frame forms its digest
@@ -398,7 +398,7 @@ __global__ void __maxnreg__(168) persistent_kernel(const __grid_constant__ PLaun
         if (blockIdx.x == 0) L.cnt->t0 = globaltimer();
     }
     __syncthreads();
-    if (digest_cta && threadIdx.x < kShaThreads<true>) {
+    if (digest_cta && threadIdx.x < kShaThreads) {
         digest_worker(L, sm, slot);
         if (threadIdx.x == 0) {
             __threadfence_block();

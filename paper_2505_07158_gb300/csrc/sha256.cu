@@ -25,12 +25,38 @@
 namespace fhd {
 namespace {
 
-// Sub-frame messages of a batch: message m is sub-frame m % n of frame m / n.
-template <bool kSplit>
-__global__ void __launch_bounds__(kShaThreads<kSplit>) sha_subframes_kernel(const __grid_constant__ Batch b) {
+// The pipelines on each pair of SMs, a bit each, sixteen to an SM (it has room for eight).  They only choose how a
+// pipeline computes (sha_pipeline); no result depends on them.
+constexpr uint32_t kSmPairs = 128;
+__device__ uint32_t g_sm_pipelines[kSmPairs];
+
+// The CTA of pipeline blockIdx.x.
+template <class Locate>
+__device__ __forceinline__ void sha_cta(Locate locate, uint32_t nmsg) {
     __shared__ ShaSmem sm;
+    __shared__ ShaShare share;
+    if (threadIdx.x == 0) {
+        uint32_t id;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
+        uint32_t *w = g_sm_pipelines + (id >> 1) % kSmPairs, bit = 0x00010001u & (id & 1 ? 0xffff0000u : 0xffffu), old = 0;
+        int k = 0;
+        for (; k < 16; ++k, bit <<= 1) {
+            old = atomicOr(w, bit);
+            if (!(old & bit)) break;
+        }
+        share.taken = w;
+        share.own = k < 16 ? bit : 0;
+        share.start = sm_pair_roomy(old | bit);
+    }
+    __syncthreads();
+    sha_pipeline<true>(locate, nmsg, blockIdx.x, threadIdx.x, 1, sm, &share);
+    if (threadIdx.x == 0) atomicAnd(share.taken, ~share.own);
+}
+
+// Sub-frame messages of a batch: message m is sub-frame m % n of frame m / n.
+__global__ void __launch_bounds__(kShaThreads, 1) sha_subframes_kernel(const __grid_constant__ Batch b) {
     const uint32_t n = b.n;
-    sha_pipeline<kSplit>(
+    sha_cta(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             if (!FHD_IN(m / n, b.count, kSiteShaDigest)) return false;
             const FrameDesc &fd = b.f[m / n];
@@ -43,15 +69,13 @@ __global__ void __launch_bounds__(kShaThreads<kSplit>) sha_subframes_kernel(cons
             out = fd.part + 32ull * i;
             return true;
         },
-        b.count * n, blockIdx.x, threadIdx.x, 1, sm);
+        b.count * n);
 }
 
 // `count` buffers of nbytes laid end to end, n sub-frames each.
-template <bool kSplit>
-__global__ void __launch_bounds__(kShaThreads<kSplit>) sha_plain_kernel(const uint8_t *data, uint64_t nbytes, uint32_t n,
-                                                                uint32_t count, uint8_t *part) {
-    __shared__ ShaSmem sm;
-    sha_pipeline<kSplit>(
+__global__ void __launch_bounds__(kShaThreads, 1) sha_plain_kernel(const uint8_t *data, uint64_t nbytes, uint32_t n,
+                                                            uint32_t count, uint8_t *part) {
+    sha_cta(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             const uint32_t k = m / n, i = m % n;
             const uint64_t lo = (uint64_t)(((unsigned __int128)nbytes * i) / n);
@@ -62,16 +86,14 @@ __global__ void __launch_bounds__(kShaThreads<kSplit>) sha_plain_kernel(const ui
             out = part + 32ull * m;
             return true;
         },
-        count * n, blockIdx.x, threadIdx.x, 1, sm);
+        count * n);
 }
 
 // Sub-frame messages of the decrypted frames (dst) of a batch, for the
 // receiver-side check; digests go to part (n per frame).
-template <bool kSplit>
-__global__ void __launch_bounds__(kShaThreads<kSplit>) sha_dst_kernel(const __grid_constant__ Batch b) {
-    __shared__ ShaSmem sm;
+__global__ void __launch_bounds__(kShaThreads, 1) sha_dst_kernel(const __grid_constant__ Batch b) {
     const uint32_t n = b.n;
-    sha_pipeline<kSplit>(
+    sha_cta(
         [&](uint32_t m, const uint8_t *&p, uint64_t &len, uint8_t *&out) {
             if (!FHD_IN(m / n, b.count, kSiteShaDigest)) return false;
             const FrameDesc &fd = b.f[m / n];
@@ -84,7 +106,7 @@ __global__ void __launch_bounds__(kShaThreads<kSplit>) sha_dst_kernel(const __gr
             out = fd.part + 32ull * i;
             return true;
         },
-        b.count * n, blockIdx.x, threadIdx.x, 1, sm);
+        b.count * n);
 }
 
 // ok[k] = (frame k's digest recomputed from its sub-frame digests, by the batch's digest mode) == frame k's
@@ -185,20 +207,11 @@ cudaError_t noalloc_scratch(uint8_t **out) {
     return cudaSuccess;
 }
 
-// Split messages while every pipeline has an SM to itself: 16 pipelines (16 frames of 720p) take 1.07 ms split
-// and 1.19 ms unsplit.  Where two share one, the two split consumer warps of the one meet those of the other on the same
-// sub-partitions, whose integer pipe one of them already fills: 256 pipelines (1080p) take 4.30 ms split and
-// 2.76 ms unsplit.
-static bool split_messages(uint32_t units) { return units <= 152; }
-
 cudaError_t launch_sha_subframes(const Batch &b, cudaStream_t s) {
     const uint32_t msgs = b.count * b.n;
     if (!msgs) return cudaSuccess;
     const uint32_t units = (msgs + kMsgPerCta - 1) / kMsgPerCta;
-    if (split_messages(units))
-        sha_subframes_kernel<true><<<units, kShaThreads<true>, 0, s>>>(b);
-    else
-        sha_subframes_kernel<false><<<units, kShaThreads<false>, 0, s>>>(b);
+    sha_subframes_kernel<<<units, kShaThreads, 0, s>>>(b);
     note_launch();
     return cudaGetLastError();
 }
@@ -207,10 +220,7 @@ cudaError_t launch_verify(const Batch &b, uint8_t *ok, cudaStream_t s) {
     const uint32_t msgs = b.count * b.n;
     if (!msgs) return cudaSuccess;
     const uint32_t units = (msgs + kMsgPerCta - 1) / kMsgPerCta;
-    if (split_messages(units))
-        sha_dst_kernel<true><<<units, kShaThreads<true>, 0, s>>>(b);
-    else
-        sha_dst_kernel<false><<<units, kShaThreads<false>, 0, s>>>(b);
+    sha_dst_kernel<<<units, kShaThreads, 0, s>>>(b);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -224,10 +234,7 @@ cudaError_t launch_sha_plain(const uint8_t *data, uint64_t nbytes, uint32_t n, u
     const uint32_t msgs = count * n;
     if (!msgs) return cudaSuccess;
     const uint32_t units = (msgs + kMsgPerCta - 1) / kMsgPerCta;
-    if (split_messages(units))
-        sha_plain_kernel<true><<<units, kShaThreads<true>, 0, s>>>(data, nbytes, n, count, part);
-    else
-        sha_plain_kernel<false><<<units, kShaThreads<false>, 0, s>>>(data, nbytes, n, count, part);
+    sha_plain_kernel<<<units, kShaThreads, 0, s>>>(data, nbytes, n, count, part);
     note_launch();
     return cudaGetLastError();
 }

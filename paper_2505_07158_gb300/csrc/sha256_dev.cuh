@@ -77,15 +77,14 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Threads of a pipeline: the consumers (two warps with split messages, one without) and the producer warp.
-template <bool kSplit>
-constexpr uint32_t kShaThreads = kSplit ? 96 : 64;
+// Threads of a pipeline: two consumer warps and the producer warp.
+constexpr uint32_t kShaThreads = 96;
 
 // The warps of one pipeline meet at hardware barrier `id`.
-template <bool kSplit>
+template <uint32_t kThreads = kShaThreads>
 __device__ __forceinline__ void pipeline_barrier(uint32_t id) {
     __syncwarp();
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kShaThreads<kSplit>) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kThreads) : "memory");
 }
 
 // a * one + b, with one a 1 that the compiler does not know: an addition on the multiplier's pipe, for the rounds'
@@ -104,6 +103,18 @@ struct ShaSmem {
     uint4 ring[kRing][4][32];
 };
 
+// A pipeline that may share its SM (sha_pipeline): the word of the pipelines on its SM and the next, a bit each in a
+// half word to each SM, and its own bit.
+struct ShaShare {
+    uint32_t hand[8][32];   // the states handed from two lanes to one
+    uint32_t start;         // sm_pair_roomy when the pipeline came,
+    uint32_t roomy[2];      // and while each block was made, by its parity
+    uint32_t *taken;
+    uint32_t own;
+};
+// No SM of the pair has a second pipeline.
+__device__ __forceinline__ bool sm_pair_roomy(uint32_t w) { return __popc(w & 0xffffu) <= 1 && __popc(w >> 16) <= 1; }
+
 // Producer warp of a pipeline: lane = message (p, len; nothing if !active), NB blocks in all.
 //
 // Message bytes reach shared memory by cp.async, kRing - 1 blocks ahead of the block being expanded (one commit
@@ -113,9 +124,9 @@ struct ShaSmem {
 // (a select by the words of s, a byte permute that also turns the word round); blocks that reach into a piece at
 // the message's edge, and the padded tail, come by byte loads.  Byte loads throughout took such a message
 // 2300 cycles a block, longer than the rounds (241 x 317 grey, 6 sub-frames: 0.24 -> 0.18 ms).
-template <bool kSplit>
+template <bool kShared>
 __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, bool active, uint64_t nb, uint64_t NB,
-                                             uint32_t lane, uint32_t bar, ShaSmem &sm) {
+                                             uint32_t lane, uint32_t bar, ShaSmem &sm, ShaShare *share) {
     const uint32_t s = (uint32_t)reinterpret_cast<uintptr_t>(p) & 15u;
     const bool shifted = __any_sync(0xffffffffu, active && s != 0);
     const uint64_t first = s ? 1 : 0, pieces = active ? (s + len) >> 4 : 0;   // whole pieces: first .. pieces - 1
@@ -134,6 +145,8 @@ __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, boo
     for (uint64_t b = 0; b < NB; ++b) {
         // Refills the slot of block b - 1, whose bytes were consumed in the previous iteration.
         issue(b + kRing - 1);
+        uint32_t taken = 0;
+        if (kShared) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(taken) : "l"(share->taken));
         if (b < nb) {
             if (b + kPrefetchBlocks < full) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 64 * (b + kPrefetchBlocks)));
             cp_async_wait<kRing - 2>();     // blocks b and b + 1 have landed
@@ -185,21 +198,22 @@ __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, boo
                 if ((t & 3) == 3) dst[t >> 2][lane] = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
-        pipeline_barrier<kSplit>(bar);     // block b is ready; block b-1 has been consumed
+        if (kShared && lane == 0) share->roomy[b & 1] = sm_pair_roomy(taken);
+        pipeline_barrier(bar);     // block b is ready; block b-1 has been consumed
     }
-    pipeline_barrier<kSplit>(bar);         // pairs with the consumers' last wait
+    pipeline_barrier(bar);         // pairs with the consumers' last wait
     cp_async_wait<0>();
 }
 
-// 32 messages per pipeline: of its threads (rtid = 0 ..), the first one or two warps compress and the last one
+// 32 messages per pipeline: of its threads (rtid = 0 ..), the first two warps compress and the last one
 // produces W + K.  Pipeline `unit` takes messages 32 unit .. 32 unit + 31 of the nmsg messages; message m is
 // located by locate(m, p, len, out) and its digest goes to out (32 bytes); locate returns false for a message that
 // failed a range check (checked builds), which is then skipped.  `bar` is the hardware barrier id the
-// pipeline's warps use.
+// pipeline's warps use; the consumers of a pipeline with a `share` meet at bar + 1.
 //
-// What bounds a pipeline is the consumers' chain of rounds.  One lane per message (kSplit false) needs ~28 cycles
+// What bounds a pipeline is the consumers' chain of rounds.  One lane per message needs ~28 cycles
 // a round: 14 shifts, LOP3s and additions at two cycles an instruction on one pipe, the other additions on the
-// multiplier's.  With kSplit two lanes of a consumer warp share a message: lane E holds e, f, g, h and lane A holds
+// multiplier's.  Split, two lanes of a consumer warp share a message: lane E holds e, f, g, h and lane A holds
 // a, b, c, d, two rounds behind E, which needs a only four rounds later.  Both run the same instructions -- three
 // rotations by their own amounts, one choice function, two sums -- and trade their new word by one shuffle, ~23
 // cycles a round:
@@ -207,39 +221,56 @@ __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, boo
 //   A, round t:  a' = (S0(a) + Maj(a, b, c)) + (e' - d)                 e' from E; e' - d is the round's T1
 // with Ch and Maj as z ^ (e & x) and z ^ (a & x) of two words made from older ones (E: x = f ^ g, z = g; A: x =
 // b ^ c, z = b & c).
-template <bool kSplit, class Locate>
-__device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32_t rtid, uint32_t bar, ShaSmem &sm) {
+//
+// Split messages take twice the issue slots, so they pay only where a pipeline has its SM to itself: two split
+// pipelines on one SM took 1.5 times as long as two unsplit ones.  With kShared the producer looks at the word of its SM's
+// pipelines (share) once a block, and the consumers, from the first block that found another one there, go on with one
+// lane per message in the first warp; whether the others come from the same launch, from another stream's or from a launch
+// confined to a few SMs makes no difference.  The two SMs of a pair do so together: with one of them split and the
+// other not, the loops of both kinds miss the instruction cache that the two appear to share, and 153 pipelines took
+// 3.59 ms where 154 took 2.90.  Digests of 30 720p frames on k streams, k = 1, 6, 8, 12: 1.17, 1.51, 1.64, 2.41 ms;
+// always split 1.17, 1.96, 2.06, 2.95; always unsplit 1.30, 1.50, 1.61, 2.52.  Without kShared (the persistent kernel,
+// one pipeline per SM) a pipeline stays split.
+template <bool kShared, class Locate>
+__device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32_t rtid, uint32_t bar, ShaSmem &sm,
+                             ShaShare *share = nullptr) {
     const uint32_t lane = rtid & 31;
     const uint32_t one = blockDim.y;       // every launch is one-dimensional
-    const bool producer = rtid >= kShaThreads<kSplit> - 32;
     const uint8_t *p = nullptr;
     uint64_t len = 0;
     uint8_t *out = nullptr;
-    uint32_t m = unit * kMsgPerCta + lane;
+    const uint32_t m = unit * kMsgPerCta + lane;
     bool active = m < nmsg;
     if (active) active = locate(m, p, len, out);
-    uint64_t nb = active ? padded_blocks(len) : 0;
+    const uint64_t nb = active ? padded_blocks(len) : 0;
     const uint64_t NB = __reduce_max_sync(0xffffffffu, (unsigned)nb);   // < 2^32 blocks per message
-    if (producer) {
-        sha_producer<kSplit>(p, len, active, nb, NB, lane, bar, sm);
-    } else if constexpr (kSplit) {
+    if (rtid >= kShaThreads - 32) {
+        sha_producer<kShared>(p, len, active, nb, NB, lane, bar, sm, share);
+        return;
+    }
+    uint64_t b = 0;
+    bool split = !kShared || share->start != 0;
+    if (rtid < 32) sm.wk[rtid >> 4][rtid & 15][32] = make_uint4(0, 0, 0, 0);
+    pipeline_barrier(bar);                 // block 0 ready
+    ShaState st;
+    st.init();
+    if (split) {
         const bool A = rtid & 1;
-        m = unit * kMsgPerCta + (rtid >> 1);
-        active = m < nmsg;
-        nb = 0;
-        if (active) active = locate(m, p, len, out);
-        if (active) nb = padded_blocks(len);
+        const uint32_t m2 = unit * kMsgPerCta + (rtid >> 1);
+        const uint8_t *p2 = nullptr;
+        uint64_t len2 = 0;
+        uint8_t *out2 = nullptr;
+        bool active2 = m2 < nmsg;
+        if (active2) active2 = locate(m2, p2, len2, out2);
+        const uint64_t nb2 = active2 ? padded_blocks(len2) : 0;
         const uint32_t mask = A ? 0xffffffffu : 0u, sign = A ? 0xffffffffu : 1u;
         const uint32_t r0 = A ? 2 : 6, r1 = A ? 13 : 11, r2 = A ? 22 : 25;
-        uint32_t init[8];
-        sha256_init(init);
         uint32_t H[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) H[q] = A ? init[q] : init[4 + q];
+        for (int q = 0; q < 4; ++q) H[q] = A ? st.h[q] : st.h[4 + q];
         const uint32_t column = A ? 32u : rtid >> 1;   // A adds no W + K
-        if (rtid < 32) sm.wk[rtid >> 4][rtid & 15][32] = make_uint4(0, 0, 0, 0);
-        pipeline_barrier<kSplit>(bar);         // block 0 ready
-        for (uint64_t b = 0; b < NB; ++b) {
+        while (b < NB && split) {
+            if (kShared) split = share->roomy[b & 1] != 0;   // after this block
             uint32_t wk[64], first[4], traded[66];
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
@@ -269,24 +300,37 @@ __device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32
                 x = s1 ^ s2;
                 z = s2 & (s1 | ~mask);
             }
-            if (b < nb) {
+            if (b < nb2) {
                 H[0] += s0;
                 H[1] += s1;
                 H[2] += s2;
                 H[3] += s3;
             }
-            pipeline_barrier<kSplit>(bar);     // done with block b; block b+1 ready
+            pipeline_barrier(bar);         // done with block b; block b+1 ready
+            ++b;
         }
-        if (active) {
-            uint32_t *d = reinterpret_cast<uint32_t *>(out) + (A ? 0 : 4);   // 32-byte slots, 4-byte aligned
+        if (split) {
+            if (active2) {
+                uint32_t *d = reinterpret_cast<uint32_t *>(out2) + (A ? 0 : 4);   // 32-byte slots, 4-byte aligned
 #pragma unroll
-            for (int q = 0; q < 4; ++q) d[q] = bswap(H[q]);
+                for (int q = 0; q < 4; ++q) d[q] = bswap(H[q]);
+            }
+            return;
         }
-    } else {
-        ShaState st;
-        st.init();
-        pipeline_barrier<kSplit>(bar);         // block 0 ready
-        for (uint64_t b = 0; b < NB; ++b) {
+        if constexpr (kShared) {           // on with one lane per message
+#pragma unroll
+            for (int q = 0; q < 4; ++q) share->hand[A ? q : 4 + q][rtid >> 1] = H[q];
+            pipeline_barrier<64>(bar + 1);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) st.h[q] = share->hand[q][lane];
+        }
+    }
+    if constexpr (kShared) {
+        if (rtid >= 32) {
+            for (; b < NB; ++b) pipeline_barrier(bar);
+            return;
+        }
+        for (; b < NB; ++b) {
             if (b < nb) {
                 // all 64 W+K words into registers first: the rounds never wait on shared memory
                 uint32_t wk[64];
@@ -313,7 +357,7 @@ __device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32
                 st.h[0] += a; st.h[1] += bb; st.h[2] += c; st.h[3] += d;
                 st.h[4] += e; st.h[5] += f; st.h[6] += g; st.h[7] += hh;
             }
-            pipeline_barrier<kSplit>(bar);     // done with block b; block b+1 ready
+            pipeline_barrier(bar);         // done with block b; block b+1 ready
         }
         if (active) store_digest(out, st.h);
     }
