@@ -1633,7 +1633,7 @@ static int permute_one(const uint8_t *src, uint8_t *dst, uint32_t height, uint32
     cudaStream_t s = (cudaStream_t)stream;
     e = cudaMallocAsync(&d.G, N, s);
     if (e != cudaSuccess) return fail(nullptr, FHD_ERR_OOM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
-    e = timed(nullptr, encrypt ? FHD_K_ENCRYPT : FHD_K_DECRYPT, s, [&] { return fhd::launch_permute(b, encrypt, s); });
+    e = timed(nullptr, encrypt ? FHD_K_ENCRYPT : FHD_K_DECRYPT, s, [&] { return fhd::launch_permute(b, encrypt, s, true); });
     cudaFreeAsync(d.G, s);
     if (e != cudaSuccess) return fail(nullptr, FHD_ERR_CUDA, std::string("permute launch: ") + cudaGetErrorString(e));
     return FHD_OK;

@@ -237,7 +237,8 @@ cudaError_t launch_master_raw(double *state5, const uint8_t *H, uint32_t n, doub
 // holds at once).
 cudaError_t launch_keystream(const Batch &b, cudaStream_t s, bool dense = false, uint32_t warps_per_cta = 1,
                              uint32_t smem = 0);
-cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s);
+// alone: the call launches nothing before the passes.
+cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s, bool alone = false);
 // The one-trajectory route: every frame's records (one chain and one warp per frame), then D and B
 // from them.  Each frame needs f.T (traj_bytes).
 cudaError_t launch_trajectory_keystream(const Batch &b, cudaStream_t s);

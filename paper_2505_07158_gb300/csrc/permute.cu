@@ -52,12 +52,16 @@ __device__ __forceinline__ uint32_t find_frame(const Batch &b, uint32_t cta) {
     return lo;
 }
 
+// In a call of the two passes alone the second one's launch overlaps the first's end (launch_permute); its CTAs wait here.
+__device__ __forceinline__ void wait_for_first_pass() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <bool kEnc, int kT = kStripThreads>
 __global__ void __launch_bounds__(kT, strip_ctas_per_sm<kT>()) strip_kernel(const __grid_constant__ Batch b,
                                                                             uint32_t cta_base) {
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<false>(b, cta)];
+    wait_for_first_pass();
     strip_pass<kEnc>(fd, cta - fd.cta0, smem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
@@ -67,6 +71,7 @@ __global__ void __launch_bounds__(kT, row_ctas_per_sm<kT>()) row_kernel(const __
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t cta = cta_base + blockIdx.x;
     const FrameDesc &fd = b.f[find_frame<true>(b, cta)];
+    wait_for_first_pass();
     row_pass<kEnc>(fd, cta - fd.rcta0, smem, threadIdx.x, blockDim.x, [] { __syncthreads(); });
 }
 
@@ -451,7 +456,7 @@ static bool single_pass_ok(const Batch &b) {
 // pass then row pass.  (Running the two passes per group of frames, so that a group's intermediate
 // frames stay in L2 between its two passes, measured slower: the smaller launches lose more to wave
 // tails than L2 residency saves.)
-cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
+cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s, bool alone) {
     if (!b.count || !b.perm_ctas) return cudaSuccess;
     size_t ssm = 0, rsm = 0;
     for (uint32_t k = 0; k < b.count; ++k) {
@@ -487,36 +492,39 @@ cudaError_t launch_permute(const Batch &b, bool encrypt, cudaStream_t s) {
     uint32_t st, rt;
     cta_threads(b.f[big].h, b.f[big].w, b.f[big].C, &st, &rt);
     st = strip_threads(b.f[big].h, b.f[big].w, b.f[big].C, ssm);
-    // (Launching the second pass with programmatic stream serialization, so that its launch overlaps the first's end,
-    // saved 2 us of a call by itself.  It is not done: with more calls in flight than hardware queues, the pass that
-    // waits holds up the queue it shares, 12 calls of 8 720p frames on 8 queues 12.5 ms against 7.3.)
-    auto rows = [&] {
-        if (rt == 128) {
-            if (encrypt) row_kernel<true, 128><<<b.row_ctas, 128, rsm, s>>>(b, 0);
-            else row_kernel<false, 128><<<b.row_ctas, 128, rsm, s>>>(b, 0);
-        } else {
-            if (encrypt) row_kernel<true><<<b.row_ctas, kRowThreads, rsm, s>>>(b, 0);
-            else row_kernel<false><<<b.row_ctas, kRowThreads, rsm, s>>>(b, 0);
-        }
-        note_launch();
-        return cudaGetLastError();
+    // Programmatic stream serialization of the second pass hides its launch latency (no CTA of it starts before the
+    // first pass has ended): a 4K frame both ways 89 -> 83 us.  Only in a call of the two passes alone: behind the other
+    // kernels of an encryption or decryption call, with more calls in flight than hardware queues, it held the queues
+    // up, 12 calls of 8 720p frames on 8 queues 12.5 ms against 7.3 without; calls of the passes, among themselves, beside
+    // and behind such calls, lost nothing (8 to 32 streams).
+    auto launch = [&](auto *kernel, uint32_t grid, uint32_t threads, size_t smem, bool second) {
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = alone && second ? 1 : 0;
+        const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, b, 0u);
+        if (err == cudaSuccess) note_launch();
+        return err != cudaSuccess ? err : cudaGetLastError();
     };
-    auto strips = [&] {
-        if (st == 256) {
-            if (encrypt) strip_kernel<true, 256><<<b.perm_ctas, 256, ssm, s>>>(b, 0);
-            else strip_kernel<false, 256><<<b.perm_ctas, 256, ssm, s>>>(b, 0);
-        } else if (st == 1024) {
-            if (encrypt) strip_kernel<true, 1024><<<b.perm_ctas, 1024, ssm, s>>>(b, 0);
-            else strip_kernel<false, 1024><<<b.perm_ctas, 1024, ssm, s>>>(b, 0);
-        } else {
-            if (encrypt) strip_kernel<true><<<b.perm_ctas, kStripThreads, ssm, s>>>(b, 0);
-            else strip_kernel<false><<<b.perm_ctas, kStripThreads, ssm, s>>>(b, 0);
-        }
-        note_launch();
-        return cudaGetLastError();
+    auto rows = [&](bool second) {
+        if (rt == 128) return launch(encrypt ? row_kernel<true, 128> : row_kernel<false, 128>, b.row_ctas, 128, rsm, second);
+        return launch(encrypt ? row_kernel<true> : row_kernel<false>, b.row_ctas, kRowThreads, rsm, second);
     };
-    if ((e = encrypt ? rows() : strips()) != cudaSuccess) return e;
-    return encrypt ? strips() : rows();
+    auto strips = [&](bool second) {
+        if (st == 256)
+            return launch(encrypt ? strip_kernel<true, 256> : strip_kernel<false, 256>, b.perm_ctas, 256, ssm, second);
+        if (st == 1024)
+            return launch(encrypt ? strip_kernel<true, 1024> : strip_kernel<false, 1024>, b.perm_ctas, 1024, ssm, second);
+        return launch(encrypt ? strip_kernel<true> : strip_kernel<false>, b.perm_ctas, kStripThreads, ssm, second);
+    };
+    if ((e = encrypt ? rows(false) : strips(false)) != cudaSuccess) return e;
+    return encrypt ? strips(true) : rows(true);
 }
 
 }  // namespace fhd
