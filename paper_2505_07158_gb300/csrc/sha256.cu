@@ -25,8 +25,7 @@
 namespace fhd {
 namespace {
 
-// The pipelines on each pair of SMs, a bit each, sixteen to an SM (it has room for eight).  They only choose how a
-// pipeline computes (sha_pipeline); no result depends on them.
+// The pipelines on each pair of SMs.  They only choose how a pipeline computes (sha_pipeline); no result depends on them.
 constexpr uint32_t kSmPairs = 128;
 __device__ uint32_t g_sm_pipelines[kSmPairs];
 
@@ -35,22 +34,7 @@ template <class Locate>
 __device__ __forceinline__ void sha_cta(Locate locate, uint32_t nmsg) {
     __shared__ ShaSmem sm;
     __shared__ ShaShare share;
-    if (threadIdx.x == 0) {
-        uint32_t id;
-        asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
-        uint32_t *w = g_sm_pipelines + (id >> 1) % kSmPairs, bit = 0x00010001u & (id & 1 ? 0xffff0000u : 0xffffu), old = 0;
-        int k = 0;
-        for (; k < 16; ++k, bit <<= 1) {
-            old = atomicOr(w, bit);
-            if (!(old & bit)) break;
-        }
-        share.taken = w;
-        share.own = k < 16 ? bit : 0;
-        share.start = sm_pair_roomy(old | bit);
-    }
-    __syncthreads();
-    sha_pipeline<true>(locate, nmsg, blockIdx.x, threadIdx.x, 1, sm, &share);
-    if (threadIdx.x == 0) atomicAnd(share.taken, ~share.own);
+    sha_pipeline<true>(locate, nmsg, blockIdx.x, threadIdx.x, 1, sm, &share, g_sm_pipelines + (sm_id() >> 1) % kSmPairs);
 }
 
 // Sub-frame messages of a batch: message m is sub-frame m % n of frame m / n.

@@ -103,17 +103,34 @@ struct ShaSmem {
     uint4 ring[kRing][4][32];
 };
 
-// A pipeline that may share its SM (sha_pipeline): the word of the pipelines on its SM and the next, a bit each in a
-// half word to each SM, and its own bit.
+// What a pipeline that may share its SM keeps in shared memory (sha_pipeline).
 struct ShaShare {
     uint32_t hand[8][32];   // the states handed from two lanes to one
     uint32_t start;         // sm_pair_roomy when the pipeline came,
     uint32_t roomy[2];      // and while each block was made, by its parity
-    uint32_t *taken;
-    uint32_t own;
 };
+
+// The pipelines on a pair of SMs: a word with a bit each, sixteen to an SM (which has room for eight).
+__device__ __forceinline__ uint32_t sm_id() {
+    uint32_t id;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
+    return id;
+}
 // No SM of the pair has a second pipeline.
 __device__ __forceinline__ bool sm_pair_roomy(uint32_t w) { return __popc(w & 0xffffu) <= 1 && __popc(w >> 16) <= 1; }
+// Takes a bit of SM `id` (0: none is left) and says whether the pair is roomy.
+__device__ __forceinline__ uint32_t take_sm_bit(uint32_t *taken, uint32_t id, uint32_t &roomy) {
+    uint32_t bit = id & 1 ? 0x10000u : 1u, old = 0;
+    for (int k = 0; k < 16; ++k, bit <<= 1) {
+        old = atomicOr(taken, bit);
+        if (!(old & bit)) {
+            roomy = sm_pair_roomy(old | bit);
+            return bit;
+        }
+    }
+    roomy = 0;
+    return 0;
+}
 
 // Producer warp of a pipeline: lane = message (p, len; nothing if !active), NB blocks in all.
 //
@@ -126,7 +143,8 @@ __device__ __forceinline__ bool sm_pair_roomy(uint32_t w) { return __popc(w & 0x
 // 2300 cycles a block, longer than the rounds (241 x 317 grey, 6 sub-frames: 0.24 -> 0.18 ms).
 template <bool kShared>
 __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, bool active, uint64_t nb, uint64_t NB,
-                                             uint32_t lane, uint32_t bar, ShaSmem &sm, ShaShare *share) {
+                                             uint32_t lane, uint32_t bar, ShaSmem &sm, ShaShare *share,
+                                             const uint32_t *sm_pipelines) {
     const uint32_t s = (uint32_t)reinterpret_cast<uintptr_t>(p) & 15u;
     const bool shifted = __any_sync(0xffffffffu, active && s != 0);
     const uint64_t first = s ? 1 : 0, pieces = active ? (s + len) >> 4 : 0;   // whole pieces: first .. pieces - 1
@@ -146,7 +164,7 @@ __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, boo
         // Refills the slot of block b - 1, whose bytes were consumed in the previous iteration.
         issue(b + kRing - 1);
         uint32_t taken = 0;
-        if (kShared) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(taken) : "l"(share->taken));
+        if (kShared) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(taken) : "l"(sm_pipelines));
         if (b < nb) {
             if (b + kPrefetchBlocks < full) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 64 * (b + kPrefetchBlocks)));
             cp_async_wait<kRing - 2>();     // blocks b and b + 1 have landed
@@ -223,8 +241,8 @@ __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, boo
 // b ^ c, z = b & c).
 //
 // Split messages take twice the issue slots, so they pay only where a pipeline has its SM to itself: two split
-// pipelines on one SM took 1.5 times as long as two unsplit ones.  With kShared the producer looks at the word of its SM's
-// pipelines (share) once a block, and the consumers, from the first block that found another one there, go on with one
+// pipelines on one SM took 1.5 times as long as two unsplit ones.  With kShared the producer looks at the word of its SMs'
+// pipelines (sm_pipelines) once a block, and the consumers, from the first block that found another one there, go on with one
 // lane per message in the first warp; whether the others come from the same launch, from another stream's or from a launch
 // confined to a few SMs makes no difference.  The two SMs of a pair do so together: with one of them split and the
 // other not, the loops of both kinds miss the instruction cache that the two appear to share, and 153 pipelines took
@@ -233,7 +251,7 @@ __device__ __forceinline__ void sha_producer(const uint8_t *p, uint64_t len, boo
 // one pipeline per SM) a pipeline stays split.
 template <bool kShared, class Locate>
 __device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32_t rtid, uint32_t bar, ShaSmem &sm,
-                             ShaShare *share = nullptr) {
+                             ShaShare *share = nullptr, uint32_t *sm_pipelines = nullptr) {
     const uint32_t lane = rtid & 31;
     const uint32_t one = blockDim.y;       // every launch is one-dimensional
     const uint8_t *p = nullptr;
@@ -245,13 +263,15 @@ __device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32
     const uint64_t nb = active ? padded_blocks(len) : 0;
     const uint64_t NB = __reduce_max_sync(0xffffffffu, (unsigned)nb);   // < 2^32 blocks per message
     if (rtid >= kShaThreads - 32) {
-        sha_producer<kShared>(p, len, active, nb, NB, lane, bar, sm, share);
+        sha_producer<kShared>(p, len, active, nb, NB, lane, bar, sm, share, sm_pipelines);
         return;
     }
     uint64_t b = 0;
-    bool split = !kShared || share->start != 0;
+    uint32_t own = 0;
+    if (kShared && rtid == 0) own = take_sm_bit(sm_pipelines, sm_id(), share->start);   // while block 0 is made
     if (rtid < 32) sm.wk[rtid >> 4][rtid & 15][32] = make_uint4(0, 0, 0, 0);
     pipeline_barrier(bar);                 // block 0 ready
+    bool split = !kShared || share->start != 0;
     ShaState st;
     st.init();
     if (split) {
@@ -310,6 +330,7 @@ __device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32
             ++b;
         }
         if (split) {
+            if (kShared && rtid == 0) atomicAnd(sm_pipelines, ~own);
             if (active2) {
                 uint32_t *d = reinterpret_cast<uint32_t *>(out2) + (A ? 0 : 4);   // 32-byte slots, 4-byte aligned
 #pragma unroll
@@ -359,6 +380,7 @@ __device__ void sha_pipeline(Locate locate, uint32_t nmsg, uint32_t unit, uint32
             }
             pipeline_barrier(bar);         // done with block b; block b+1 ready
         }
+        if (rtid == 0) atomicAnd(sm_pipelines, ~own);
         if (active) store_digest(out, st.h);
     }
 }
