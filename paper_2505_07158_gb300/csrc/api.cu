@@ -896,6 +896,17 @@ const char *bounds_site_name(unsigned site) {
         default: return "unknown site";
     }
 }
+// 152, a GB300's, where the device does not say.
+uint32_t sm_count() {
+    static std::atomic<int> known[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    if ((n = known[dev].load(std::memory_order_relaxed)) > 0) return (uint32_t)n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 152;
+    known[dev].store(n, std::memory_order_relaxed);
+    return (uint32_t)n;
+}
+
 }  // namespace fhd
 
 extern "C" {

@@ -140,6 +140,8 @@ struct PLaunch {
     PSide s[2];
 };
 
+uint32_t sm_count();   // SMs of the current device (api.cu)
+
 cudaError_t launch_persistent(const PLaunch &L, size_t mem_smem, cudaStream_t s);
 size_t persistent_mem_smem_limit();   // shared memory the permutation tasks of a persistent launch may use
 uint32_t persistent_mem_threads();    // and the threads they run on

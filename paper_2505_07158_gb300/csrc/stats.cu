@@ -263,7 +263,7 @@ __global__ void npcr_finish_kernel(const unsigned long long *acc, uint32_t items
 // CTA per (frame, direction) walked 40 pairs a thread one after another on 90 of the 152 SMs.  The pairs are now
 // shared by the CTAs of a cluster, kLoads a thread at a time, and the sums meet in its first CTA's hands through
 // distributed shared memory, with no counters to clear and no second launch.  10,000 pairs in each direction of 30
-// frames: 57 -> 32 us.  A thread has at most 2^22 / 256 pairs, whose sums of squares
+// frames: 57 -> 27 us.  A thread has at most 2^22 / 256 pairs, whose sums of squares
 // fit 32 bits.
 template <int C>
 __global__ void __launch_bounds__(kStatThreads) corr_kernel(const uint8_t *frames, uint32_t h, uint32_t w,
@@ -355,8 +355,15 @@ __global__ void __launch_bounds__(kStatThreads) corr_kernel(const uint8_t *frame
 template <int C>
 cudaError_t corr_launch(const uint8_t *frames, uint32_t count, uint32_t h, uint32_t w, const uint32_t *pairs,
                         uint32_t npairs, long long *sums, double *out, unsigned *status, cudaStream_t s) {
-    // one CTA up to where its threads have their loads in flight at once, and where the grid could not hold eight
-    const uint32_t parts = npairs <= 4 * kStatThreads || count > (1u << 24) ? 1 : 8;
+    // CTAs to an item: twice as many while its pairs keep their threads in loads (1,024 pairs a CTA), and the items have no
+    // more than three CTAs to an SM, or ten where a CTA keeps 3,500 pairs; a CTA more costs ~6 ns.  Eight throughout took
+    // 176 us for 1,025 pairs of 1,000 frames, 33 with one; by this rule 10,000 pairs of 30, 60, 200 and 300 frames take
+    // 27, 43, 87 and 64 us (eight: 31, 46, 110, 111; one: 41, 53, 122, 64).
+    const uint64_t items = 3ull * count, sms = sm_count();
+    uint32_t parts = 1;
+    while (parts < 8 && npairs > 1024 * parts &&
+           (items * 2 * parts <= 3 * sms || (items * 2 * parts <= 10 * sms && npairs / (2 * parts) >= 3500)))
+        parts *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(count * 3 * parts);
     cfg.blockDim = dim3(kStatThreads);

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import paper_2505_07158_gb300 as fhd
+from paper_2505_07158_gb300 import _lib
 
 pytestmark = pytest.mark.gpu
 
@@ -84,3 +85,33 @@ def test_digest_time_of_pipelines_that_share_an_sm():
     S = [torch.cuda.Stream() for _ in X]
     t = [fastest(lambda: digests(X[:n], S[:n])) for n in (1, 2)]
     assert t[1] < 1.45 * t[0], t
+
+
+def pairs_of(count, h, w, npairs):
+    g = torch.Generator(device="cuda").manual_seed(npairs)
+    return torch.stack([torch.randint(0, h - 1, (count, 3, npairs), device="cuda", generator=g),
+                        torch.randint(0, w - 1, (count, 3, npairs), device="cuda", generator=g)], dim=-1).int()
+
+
+def test_correlation_time_of_many_frames():
+    """1,025 pairs of each of 1,000 frames against 1,024: the pairs of a direction are not spread over more CTAs where the
+    frames fill the GPU by themselves (equal; 5 times where they were)."""
+    a = noise(1000, 32, 32, 3)
+    pairs = [pairs_of(1000, 32, 32, n) for n in (1024, 1025)]
+    t = [fastest(lambda: [_lib.fhd_stats_correlation(a, p) for _ in range(10)]) for p in pairs]
+    assert t[1] < 1.5 * t[0], t
+
+
+@pytest.mark.parametrize("count,npairs", [(1, 1025), (1, 2049), (1, 4097), (30, 10000), (51, 7000), (100, 2048), (180, 7000)])
+def test_correlation_sums_by_any_number_of_ctas(count, npairs):
+    """Two, four and eight CTAs to a frame's direction, and one: exact sums."""
+    h, w = 37, 53
+    a, p = noise(count, h, w, 3, seed=count), pairs_of(count, h, w, npairs)
+    sums, _, status = _lib.fhd_stats_correlation(a, p)
+    assert int(status) == 0
+    f = torch.arange(count, device="cuda")[:, None]
+    for d, (di, dj) in enumerate(((0, 1), (1, 0), (1, 1))):
+        i, j = p[:, d, :, 0].long(), p[:, d, :, 1].long()
+        x, y = a[f, i, j].long(), a[f, i + di, j + dj].long()
+        ref = torch.stack([x.sum(1), y.sum(1), (x * x).sum(1), (y * y).sum(1), (x * y).sum(1)], dim=-1)
+        assert torch.equal(sums[:, :, d], ref)
