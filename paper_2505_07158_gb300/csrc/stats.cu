@@ -387,8 +387,8 @@ cudaError_t corr_launch(const uint8_t *frames, uint32_t count, uint32_t h, uint3
 // z log2 z, ~30 binary64 instructions each, held the binary64 pipes for most
 // of the rest.  The bytes are now read kLoads to a thread at a time whatever
 // the row, and a term is computed once for each count that occurs up to 256
-// (the counts of a block are small: the largest of the 900 noise blocks of
-// 44 x 44 in 30 frames is under 32, one warp's work).  Those 900 blocks: 82 -> 22 us.
+// (the counts of a noise block of 44 x 44 are under 32, one warp's work; a flat
+// block's one count is a warp's work too).  900 noise blocks of 44 x 44: 82 -> 22 us.
 template <int C>
 __global__ void __launch_bounds__(kStatThreads) block_entropy_kernel(const uint8_t *frames, uint32_t h, uint32_t w,
                                                                      const uint32_t *blocks, uint32_t k, uint32_t bs,
@@ -396,14 +396,14 @@ __global__ void __launch_bounds__(kStatThreads) block_entropy_kernel(const uint8
     constexpr int kLoads = 8;
     __shared__ uint32_t hist[C][256];
     __shared__ double term[256];   // of count z in term[z - 1]
-    __shared__ uint32_t largest;
+    __shared__ bool occurs[256];   // whether a bin has that count
     const uint32_t f = blockIdx.x / k, q = blockIdx.x % k;
     const uint8_t *F = frames + (uint64_t)f * h * w * C;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t r0 = blocks[2 * ((uint64_t)f * k + q)], c0 = blocks[2 * ((uint64_t)f * k + q) + 1];
     const bool inside = r0 <= h - bs && c0 <= w - bs;   // bs <= h, w
     for (uint32_t t = threadIdx.x; t < C * 256; t += kStatThreads) (&hist[0][0])[t] = 0;
-    if (threadIdx.x == 0) largest = 0;
+    occurs[threadIdx.x] = false;
     __syncthreads();
     if (inside) {
         const uint32_t row = bs * C, down = kStatThreads / row, along = kStatThreads % row;
@@ -434,13 +434,13 @@ __global__ void __launch_bounds__(kStatThreads) block_entropy_kernel(const uint8
         atomicOr(status, 1u);
     }
     __syncthreads();
-    uint32_t z = 0;
 #pragma unroll
-    for (int c = 0; c < C; ++c) z = max(z, hist[c][threadIdx.x]);
-    z = __reduce_max_sync(0xffffffffu, z);
-    if (lane == 0) atomicMax(&largest, z);
+    for (int c = 0; c < C; ++c) {
+        const uint32_t z = hist[c][threadIdx.x];
+        if (z - 1 < 256) occurs[z - 1] = true;
+    }
     __syncthreads();
-    if (threadIdx.x < largest) term[threadIdx.x] = (double)(threadIdx.x + 1) * log2((double)(threadIdx.x + 1));
+    if (occurs[threadIdx.x]) term[threadIdx.x] = (double)(threadIdx.x + 1) * log2((double)(threadIdx.x + 1));
     __syncthreads();
     if (warp < C) {
         double e = 0.0;

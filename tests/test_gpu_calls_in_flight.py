@@ -115,3 +115,14 @@ def test_correlation_sums_by_any_number_of_ctas(count, npairs):
         x, y = a[f, i, j].long(), a[f, i + di, j + dj].long()
         ref = torch.stack([x.sum(1), y.sum(1), (x * x).sum(1), (y * y).sum(1), (x * y).sum(1)], dim=-1)
         assert torch.equal(sums[:, :, d], ref)
+
+
+def test_local_entropy_time_of_flat_blocks():
+    """100 blocks of 16 x 16 of each of 300 flat frames against noise frames: a flat block has one logarithm to take, a
+    noise block a dozen (no dearer; 1.75 times where every count up to the largest
+    had its logarithm)."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    blocks = torch.randint(0, 49, (300, 100, 2), device="cuda", generator=g).int()
+    rough = noise(300, 64, 64, 3)
+    t = [fastest(lambda: _lib.fhd_stats_local_entropy(a, blocks, 16)) for a in (rough, torch.zeros_like(rough))]
+    assert t[1] < 1.4 * t[0], t
