@@ -374,10 +374,12 @@ __device__ __forceinline__ void int_constants(IntVar &s, IntLane &L, int lane, d
     if (lane < 4 * kIntChains && (lane & 3) >= 2) L.fo1 = (lane & 3) == 2 ? fb : fg;
 }
 
-// gamma as a factor: its exponent within the shifts' range and its low 26 bits not all zero.
+// gamma as a factor: its exponent within the shifts' range and its low 26 bits not all zero.  A positive gamma from 1/4 on
+// is left to binary64: its chains leave the ranges before long (and overflow in the end), and every step is then marked,
+// 2,048 steps at gamma = 0.9 3.80 ms against 2.11 (0.3: 2.35).
 __device__ __forceinline__ bool int_gamma_ok(double gamma) {
     int n0, n1, e;
-    return split_double(gamma, false, n0, n1, e) && e >= -8 && e <= 0 && ((uint32_t)n0 << 6) != 0;
+    return split_double(gamma, false, n0, n1, e) && e >= -8 && e <= (gamma > 0.0 ? -3 : 0) && ((uint32_t)n0 << 6) != 0;
 }
 
 // Constants of this lane.
