@@ -120,6 +120,11 @@ __global__ void __launch_bounds__(32, 1) keystream_pair_kernel(const __grid_cons
 // per CTA took 3 % longer, with 608 pairs too); beyond, its one pair per warp would cost more issue slots than the
 // binary64 kernel's three have pipe time.
 constexpr uint32_t kPairLaunch = 608;
+// Fewest steps of its longest slice, from nine pairs on: iterates from anywhere (Algorithm 2) need some steps to come to
+// the attractor, and many a step on the way is marked; a launch takes as long as its unluckiest pair.  32 pairs and
+// more of ~11, 21 and 43 steps: 23, 38, 56-59 us here, 19, 31, 56 in the binary64 kernel; one pair of 21 steps 33 and
+// 42, eight 32 and 35.
+constexpr uint64_t kPairSteps = 48, kFewPairs = 8;
 
 // K2t: the records of one frame per warp, its chain in lanes 0..3.
 __global__ void __launch_bounds__(32 * kIntWarps, 1) trajectory_kernel(const __grid_constant__ Batch b) {
@@ -285,7 +290,13 @@ cudaError_t launch_keystream(const Batch &b, cudaStream_t s, bool dense, uint32_
         note_launch();
         return cudaGetLastError();
     }
-    if (k == 1 && smem == 0 && b.count * b.n <= kPairLaunch) {
+    uint64_t steps = 0;
+    for (uint32_t f = 0; f < b.count; ++f) {
+        const FrameDesc &d = b.f[f];
+        const uint64_t LD = (uint64_t)d.C * (d.h + d.w);
+        steps = std::max(steps, (2 * ((LD + b.n - 1) / b.n) + (d.N + b.n - 1) / b.n + 23) / 24);
+    }
+    if (k == 1 && smem == 0 && b.count * b.n <= kPairLaunch && (steps >= kPairSteps || b.count * b.n <= kFewPairs)) {
         keystream_pair_kernel<<<b.count * b.n, 32, 0, s>>>(b);
         note_launch();
         return cudaGetLastError();

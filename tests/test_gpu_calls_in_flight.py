@@ -1,10 +1,12 @@
 """What calls cost beside other calls, and on inputs that a fast path does not suit: ratios of times within one process
-(the fastest of several passes), each with at least a quarter between the bar and what either side of it measures."""
+(the fastest of several passes), each with a bar between what the call takes and what it took where it went wrong."""
 import hashlib
 
+import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2505_07158_gb300 as fhd
 from paper_2505_07158_gb300 import _lib
 
@@ -137,3 +139,26 @@ def test_chain_time_at_gammas_beyond_the_attractors():
         st = torch.tensor([12.3, 4.5, 23.4, 7.8, gamma], dtype=torch.float64, device="cuda")
         t.append(fastest(lambda: fhd.fhd_master(st, H, n_workers=1024)))
     assert t[1] < 1.25 * t[0], t
+
+
+def test_worker_pair_time_of_short_slices():
+    """304 pairs of 21 steps each from iterates off the attractor against 305 x 2, which the binary64 kernel takes: as
+    long (1.06 times; 1.28 where the short slices took the integer step)."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    scale = torch.tensor([20.0, 20.0, 40.0, 20.0], dtype=torch.float64, device="cuda")
+    t = []
+    for n in (610, 304):
+        IR = torch.rand((2 * n, 4), dtype=torch.float64, device="cuda", generator=g) * scale
+        t.append(fastest(lambda: [fhd.fhd_keystream(IR, -0.9123, n, 500, 1, n_workers=n) for _ in range(30)]))
+    assert t[1] < 1.15 * t[0], t
+
+
+@pytest.mark.parametrize("n,w", [(1, 23), (8, 23), (9, 23), (9, 1140), (9, 1150), (32, 1100), (32, 1200), (304, 1150), (608, 1150)])
+def test_worker_pairs_on_both_sides_of_the_short_slices(n, w):
+    """Few pairs and many, slices of one step and on both sides of 48, against the oracle."""
+    g = np.random.default_rng(n + w)
+    IR = g.uniform(0, 1, (2 * n, 4)) * [20, 20, 40, 20]
+    D_ref, B_ref = oracle.keystream(IR, -0.9123, n, w, 1, n, 0.01)
+    D, B = fhd.fhd_keystream(torch.from_numpy(IR).cuda(), -0.9123, n, w, 1, n_workers=n)
+    assert np.array_equal(D.cpu().numpy().view(np.uint16), D_ref)
+    assert np.array_equal(B.cpu().numpy().reshape(-1), np.asarray(B_ref).reshape(-1))
