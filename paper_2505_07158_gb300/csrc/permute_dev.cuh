@@ -76,16 +76,16 @@ __device__ __forceinline__ void transpose4x4(uint32_t &a, uint32_t &b, uint32_t 
 //   transposed back into four row words by selectors that undo the swizzle.
 // Every global access is a 32-bit word per thread, consecutive across the threads of a row quad.
 //
-// Off: the type of offsets into the frame (32 bits below 4 GB).  What bounds the pass is latency, 96 bytes of a
-// row at a time: the strip fills the SM, so its two phases do not overlap.  The instructions were next, 218 a quad with
-// 64-bit offsets formed for each access and eight shared loads with their indices, and half that now.  A 4K frame
+// Offsets into the frame take 32 bits (a frame is at most 12,288 x 16,384 x 4 bytes).  What bounds the pass is latency,
+// 96 bytes of a row at a time: the strip fills the SM, so its two phases do not overlap.  The instructions were next, 218 a
+// quad with 64-bit offsets formed for each access and eight shared loads with their indices, and half that now.  A 4K frame
 // by itself, both passes: encrypt 51.4 -> 44.5 us, decrypt 53.8 -> 48.9 us, with CTAs of 1024 threads.
-template <bool kEnc, bool kL2, class Off, class Sync>
+template <bool kEnc, bool kL2, class Sync>
 __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uint8_t *smem, uint32_t tid,
                               uint32_t nthr, Sync sync) {
     constexpr uint32_t kU = 2;   // row quads per thread and batch: 8 independent 32-bit loads in flight, B's one batch ahead
     const uint32_t h = fd.h, w = fd.w, C = fd.C, H4 = h >> 2, NL = QC >> 2;
-    const Off row = (Off)w * C;
+    const uint32_t row = w * C;
     const uint8_t *src = kEnc ? fd.G : fd.src, *key = fd.B;
     uint8_t *out = kEnc ? fd.dst : fd.G;
     uint32_t *S = reinterpret_cast<uint32_t *>(smem);
@@ -94,10 +94,10 @@ __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uin
     const uint32_t LT = NL <= 16 ? 16 : (NL + 31) & ~31u, lam = tid % LT, p0 = tid / LT, nq = nthr / LT;
     const uint32_t x = (QC & 31 ? lam >> 2 : lam >> 3) & 3;
     const bool live = lam < NL && p0 < nq;
-    const Off at0 = (Off)j0 * C + 4 * lam;   // this column quad in a row
+    const uint32_t at0 = j0 * C + 4 * lam;   // this column quad in a row
     // column m's rotation: whole row quads, and the byte selector of the rest
     uint32_t a[4], sel[4];
-    auto load = [&](const uint8_t *p, Off at) -> uint32_t {
+    auto load = [&](const uint8_t *p, uint32_t at) -> uint32_t {
         return FHD_IN(at + 3, fd.N, kSiteStripLoad) ? pass_ld<kL2>(reinterpret_cast<const uint32_t *>(p + at)) : 0;
     };
     if (live) {
@@ -115,7 +115,7 @@ __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uin
         }
         for (uint32_t k0 = p0 * kU; k0 < H4; k0 += nq * kU) {
             uint32_t v[kU][4];
-            Off at = at0 + (Off)(4 * k0) * row;
+            uint32_t at = at0 + (4 * k0) * row;
 #pragma unroll
             for (uint32_t u = 0; u < kU; ++u)
 #pragma unroll
@@ -148,7 +148,7 @@ __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uin
     }
     uint32_t kb[kU][4];   // B words of a batch's output rows (encrypt)
     auto load_key = [&](uint32_t t0) {
-        Off at = at0 + (Off)(4 * t0) * row;
+        uint32_t at = at0 + (4 * t0) * row;
 #pragma unroll
         for (uint32_t u = 0; u < kU; ++u)
 #pragma unroll
@@ -174,7 +174,7 @@ __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uin
         return FHD_IN(i + 3, words, kSiteStripSmem) ? *reinterpret_cast<const uint4 *>(S + i) : make_uint4(0, 0, 0, 0);
     };
     for (uint32_t t0 = p0 * kU; t0 < H4; t0 += nq * kU) {
-        const Off first = at0 + (Off)(4 * t0) * row;
+        const uint32_t first = at0 + (4 * t0) * row;
         uint32_t kc[kU][4];
         if (kEnc && kL2) load_key(t0);
         if (kEnc) {
@@ -185,7 +185,7 @@ __device__ void strip_pass_cw(const FrameDesc &fd, uint32_t j0, uint32_t QC, uin
         }
         if (kEnc && !kL2) load_key(t0 + nq * kU);
         uint4 before = quad(t0 ? t0 - 1 : H4 - 1);
-        Off at = first;
+        uint32_t at = first;
 #pragma unroll
         for (uint32_t u = 0; u < kU; ++u) {
             if (t0 + u >= H4) break;
@@ -234,10 +234,7 @@ __device__ void strip_pass(const FrameDesc &fd, uint32_t strip, uint8_t *smem, u
         // memory holds it without padding)
         if ((h & 3) == 0 && (QC & 3) == 0 && rowB % 4 == 0 && base % 4 == 0 && nthr >= QC / 4 && aligned(src, 4) &&
             aligned(out, 4) && aligned(fd.B, 4)) {
-            if (fd.N <= 0xffffffffu)
-                strip_pass_cw<kEnc, kL2, uint32_t>(fd, j0, QC, smem, tid, nthr, sync);
-            else
-                strip_pass_cw<kEnc, kL2, uint64_t>(fd, j0, QC, smem, tid, nthr, sync);
+            strip_pass_cw<kEnc, kL2>(fd, j0, QC, smem, tid, nthr, sync);
             return;
         }
     }
