@@ -115,11 +115,11 @@ __global__ void __launch_bounds__(32, 1) keystream_pair_kernel(const __grid_cons
     if (f >= b.count) return;
     keystream_warp<1>(b.f[f], b.n, Rk4{b.hstep, b.hhalf, b.hsixth}, pg, threadIdx.x, &b.tab);
 }
-// Most worker pairs of a launch of it: one warp per sub-partition of the GPU (152 SMs).  Up to there a pair's
+// Most worker pairs of a launch of it: one warp per sub-partition of the GPU (608 on 152 SMs).  Up to there a pair's
 // latency is the launch's (32 pairs of a 720p frame: 2.91 ms against 4.23 ms for the binary64 kernel; four pairs
 // per CTA took 3 % longer, with 608 pairs too); beyond, its one pair per warp would cost more issue slots than the
 // binary64 kernel's three have pipe time.
-constexpr uint32_t kPairLaunch = 608;
+uint32_t pair_launch() { return 4 * sm_count(); }
 // Fewest steps of its longest slice, from nine pairs on: iterates from anywhere (Algorithm 2) need some steps to come to
 // the attractor, and many a step on the way is marked; a launch takes as long as its unluckiest pair.  32 pairs and
 // more of ~11, 21 and 43 steps: 23, 38, 56-59 us here, 19, 31, 56 in the binary64 kernel; one pair of 21 steps 33 and
@@ -296,7 +296,7 @@ cudaError_t launch_keystream(const Batch &b, cudaStream_t s, bool dense, uint32_
         const uint64_t LD = (uint64_t)d.C * (d.h + d.w);
         steps = std::max(steps, (2 * ((LD + b.n - 1) / b.n) + (d.N + b.n - 1) / b.n + 23) / 24);
     }
-    if (k == 1 && smem == 0 && b.count * b.n <= kPairLaunch && (steps >= kPairSteps || b.count * b.n <= kFewPairs)) {
+    if (k == 1 && smem == 0 && b.count * b.n <= pair_launch() && (steps >= kPairSteps || b.count * b.n <= kFewPairs)) {
         keystream_pair_kernel<<<b.count * b.n, 32, 0, s>>>(b);
         note_launch();
         return cudaGetLastError();

@@ -483,9 +483,9 @@ cudaError_t launch_stats_histogram(const uint8_t *frames, uint32_t count, uint64
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(hist_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 131072);
     if (e != cudaSuccess) return e;
-    // CTAs of 32 C KB of counters and 512 threads, at most four of them to an SM, on 152 SMs; a run of 64 KB at least,
+    // CTAs of 32 C KB of counters and 512 threads, at most four of them to an SM; a run of 64 KB at least,
     // for the sum of the copies
-    const uint32_t cuts = stat_cuts(frame_bytes, count, C, 152 * std::min(4u, 227u / (32 * C + 1)), 1u << 16, 1u << 20);
+    const uint32_t cuts = stat_cuts(frame_bytes, count, C, sm_count() * std::min(4u, 227u / (32 * C + 1)), 1u << 16, 1u << 20);
     const uint64_t ctas = (uint64_t)cuts * count;
     switch (C) {
         case 1: hist_kernel<1><<<(unsigned)ctas, kHistThreads, smem, s>>>(frames, total, frame_bytes, cuts, hist64); break;
@@ -506,7 +506,7 @@ cudaError_t launch_stats_npcr(const uint8_t *a, const uint8_t *b, uint32_t count
     zero_kernel<<<zero_grid(items * 2), 256, 0, s>>>(acc, items * 2);
     note_launch();
     // eight CTAs of 256 threads to an SM; runs of 64 KB where there are more than a round of them
-    const uint32_t cuts = stat_cuts(frame_bytes, count, C, 152 * 8, 1u << 13, 1u << 16);
+    const uint32_t cuts = stat_cuts(frame_bytes, count, C, sm_count() * 8, 1u << 13, 1u << 16);
     const unsigned grid = cuts * count;
     switch (C) {
         case 1: npcr_kernel<1><<<grid, kStatThreads, 0, s>>>(a, b, total, frame_bytes, cuts, acc); break;
