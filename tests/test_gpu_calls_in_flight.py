@@ -162,3 +162,14 @@ def test_worker_pairs_on_both_sides_of_the_short_slices(n, w):
     D, B = fhd.fhd_keystream(torch.from_numpy(IR).cuda(), -0.9123, n, w, 1, n_workers=n)
     assert np.array_equal(D.cpu().numpy().view(np.uint16), D_ref)
     assert np.array_equal(B.cpu().numpy().reshape(-1), np.asarray(B_ref).reshape(-1))
+
+
+def test_chain_time_on_the_attractor():
+    """The integer step is what runs, and few of its steps are done again: 2,048 steps at gamma = -0.9123 against -1, which
+    it does not take (0.68 times)."""
+    H = noise(32)
+    t = []
+    for gamma in (-1.0, -0.9123):
+        st = torch.tensor([12.3, 4.5, 23.4, 7.8, gamma], dtype=torch.float64, device="cuda")
+        t.append(fastest(lambda: fhd.fhd_master(st, H, n_workers=1024)))
+    assert t[1] < 0.8 * t[0], t

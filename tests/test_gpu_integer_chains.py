@@ -41,3 +41,14 @@ def test_worker_pairs_that_leave_the_ranges(gamma, scale):
     D_ref, B_ref = oracle.keystream(IR, gamma, 60, 100, 3, 4, 0.01)
     D, B = fhd.fhd_keystream(torch.from_numpy(IR).cuda(), gamma, 60, 100, 3, n_workers=4)
     assert np.array_equal(D.cpu().numpy().view(np.uint16), D_ref) and np.array_equal(B.cpu().numpy().reshape(-1), np.asarray(B_ref).reshape(-1))
+
+
+@pytest.mark.parametrize("gamma,h", [(-0.9123, 8.1e-4), (-0.0041, 8.1e-4), (0.2499, 8.1e-4), (-1.9999, 8.1e-4), (-0.9123, 0.02),
+                                     (-1.52, 0.0399), (-0.9123, 0.0399), (-0.0601, 0.0399), (-1.9999, 0.0399), (-0.0041, 0.01),
+                                     (0.0041, 0.01), (-1.9999, 0.01), (-0.06, 0.01)])
+@pytest.mark.parametrize("seed", range(2))
+def test_master_chains_at_the_ends_of_the_integer_steps_range(gamma, h, seed):
+    """Step sizes and gammas just inside the range that the integer step takes: its shadows' error bounds scale with both,
+    and a bound that is too small shows in a rare step only."""
+    g = np.random.default_rng(100 + seed)
+    check_master(g.uniform(-50, 50, 4), gamma, 1024, h, seed)
