@@ -161,8 +161,8 @@ int g_ks_route = FHD_KS_ROUTE_TRAJECTORY;
 
 }  // namespace
 
-// Error bounds of the integer step's shadows (lorenz_int.cuh), unscaled, for |x|, |y| < 32, |z| < 64, |w| < 256
-// and |gamma| < 2: interval arithmetic over the stages with u = 2^-24 the rounding unit of a float.  A state's
+// Error bounds of the integer step's shadows (lorenz_int.cuh), unscaled, for |x| < 28, |y| < 30, |z| < 50, |w| < 216 (the
+// ranges that every unmarked step keeps to) and |gamma| < 2: interval arithmetic over the stages with u = 2^-24 the rounding unit of a float.  A state's
 // shadow is off by less than 2^-23 of its range; a stage's by that, plus c times the error of k, plus roundings.
 // All bounds are taken over the four stages and widened by a quarter.
 IntStepTab int_step_tab(double h) {

@@ -460,12 +460,12 @@ __device__ void keystream_warp(const FrameDesc &fd, uint32_t n, const Rk4 &c, ui
 // The records of one frame per chain of the warp, in the six-chain layout of LHCS_m (lane 4c + v holds
 // variable v of chain c; lanes 24..31 hold the constants).  fd: this lane's frame (the four lanes of a chain
 // share it), nullptr where the chain has none (the launches give a warp one chain; past two of them the warp steps
-// in binary64).  Steps k = 1, 2, ... take the state from s_k to s_{k+1}: while k < 2n it is LHCS_m's iterate IR[k], read back, and from k = 2n on one RK4 step.  After step k >= 2
-// the warp writes record k - 2 = (s_k, s_{k+1}): each lane the 48-bit XOR of its variable's two bit patterns
-// (the six low mantissa bytes) as three 16-bit words, which needs no exchange between the lanes: a shuffle that
-// reads a fresh binary64 result, as the earlier packing into 64-bit words did, cost ~100 cycles a step.  A chain
-// is strictly sequential, so its time is the number of steps times the step's latency; the warp runs to its
-// longest frame.  All 32 lanes call it together.
+// in binary64).  Steps k = 1, 2, ... take the state from s_k to s_{k+1}: while k < 2n it is LHCS_m's iterate IR[k],
+// read back, and from k = 2n on one RK4 step.  After step k >= 2 the warp writes record k - 2 = (s_k, s_{k+1}): each
+// lane the 48-bit XOR of its variable's two bit patterns (the six low mantissa bytes) as three 16-bit words, which
+// needs no exchange between the lanes: a shuffle that reads a fresh binary64 result, as the earlier packing into
+// 64-bit words did, cost ~100 cycles a step.  A chain is strictly sequential, so its time is the number of steps
+// times the step's latency; the warp runs to its longest frame.  All 32 lanes call it together.
 __device__ void trajectory_warp(const FrameDesc *fd, uint32_t n, const Rk4 &c, const IntStepTab &tab, int lane) {
     const int v = lane & 3;
     const bool active = fd != nullptr && lane < 4 * kChainsPerWarp;

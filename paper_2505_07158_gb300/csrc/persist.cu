@@ -8,7 +8,7 @@
 //     per task, largest frames first); the pipeline that completes a frame's messages folds (Algorithm 1)
 //     or tree-hashes them into the frame digest and publishes it;
 //   * warps 2, 3 and 5: chain workers, one on each of sub-partitions 1-3, so that a chain has its
-//     sub-partition's binary64 pipe, and its issue port, to itself; per frame, smallest first
+//     sub-partition's pipes and its issue port to itself; per frame, smallest first
 //     (the order in which their digests arrive): the LHCS_m task of every stream whose earliest frame it
 //     is (Algorithm 1), then the frame's keystream tasks (Algorithm 2, the two sides interleaved): with the
 //     one-trajectory route one task per frame and side, the frame's trajectory records (traj_records in
@@ -50,7 +50,9 @@ __device__ __forceinline__ int chain_index(uint32_t warp) { return warp == 2 ? 0
 __device__ __forceinline__ uint32_t mem_index(uint32_t warp) { return warp == 4 ? 0 : warp - 5; }   // warps 4, 6..11
 constexpr unsigned kBarSha = 1, kBarMem = 2;
 // Shared memory: digests of the chain workers, broadcast slots and flag; then the digest pipeline's and, from
-// kPMemOffset, the permutation group's, which overlap: in a CTA with a pipeline the group starts after it.
+// kPMemOffset, the permutation group's, which overlap: in a CTA with a pipeline the group starts after it.  From there
+// on the group has 207,696 bytes, room for a 4K frame's strips of 32 pixels (207,360), which the pipeline's end (25,264)
+// would not leave.
 constexpr size_t kPHeadSmem = 32 * kChainWarps + 64 + 16, kPMemOffset = 24752;
 constexpr size_t kPSmemLimit = 232448;
 static_assert(kPHeadSmem % 16 == 0 && kPMemOffset % 16 == 0 && kPHeadSmem <= kPMemOffset, "16-byte aligned parts");
@@ -268,7 +270,7 @@ __device__ void chain_worker(const PLaunch &L, uint8_t *H) {
     }
 }
 
-// ---- permutation group (warps 6-17)
+// ---- permutation group (warps 4 and 6-11)
 __device__ void mem_worker(const PLaunch &L, uint8_t *smem, unsigned *slot) {
     const uint32_t mtid = 32 * mem_index(threadIdx.x >> 5) + (threadIdx.x & 31);
     auto sync = [] { bar_sync(kBarMem, kMemThreads); };
