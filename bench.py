@@ -250,7 +250,10 @@ def traj_steps(h, w, C, n):
     return R + 2 - 2 * n
 
 
-RK4_CHAIN_CYCLES = 1040  # dependency chain of one RK4 step on the integer pipes: four stages of ~260 cycles
+# Dependency chain of one RK4 step on the integer pipes: four stages of ~260 cycles (exchange 50, product 50, sum 30, k 30,
+# product 50, next input 50).  An estimate from the instructions' latencies, not a measurement.
+RK4_CHAIN_CYCLES = 1040
+RK4_FP64_INSTR = 27     # binary64 instructions of the same step in binary64
 
 
 def sha_blocks(N, n):
@@ -755,9 +758,11 @@ def run_ours(args):
     def traj_roof(k):
         # One chain per frame, strictly sequential: the launch lasts its longest chain, one warp's RK4 steps on
         # the integer pipes.  achieved = its steps per second (launch time alone), peak = the steps per second of
-        # the step's dependency chain at the sampled clock: frac is how much of the launch that chain takes (the
-        # rest is the warp's issue and the steps done again in binary64).  The whole GPU's binary64 fraction
-        # (algorithmic ops of all launches over the union of their spans) is reported beside it.
+        # the step's dependency chain at the sampled clock, as estimated (RK4_CHAIN_CYCLES): frac is how much of the
+        # launch that chain would take (the rest is the warp's issue and the steps done again in binary64).  Beside it
+        # the measured yardsticks: the rate of the same step's binary64 instructions at the probe's rate of one
+        # sub-partition (which the integer step is there to pass), and the whole GPU's binary64 fraction
+        # (algorithmic ops of all launches over the union of their spans).
         steps = traj_steps(HGT, WID, CH, N_WORKERS)
         ms = alone[k][0] / alone[k][1]
         mhz = clocks_mhz or 2070.0
@@ -766,7 +771,9 @@ def run_ours(args):
         gpu_ach = n_l * steps * per_step_frames * RK4_FP64_OPS / (busy_ms(k) / 1000.0) / 1e12
         return {"bound": "latency", "achieved": ach, "peak": peak, "unit": "RK4 steps/s of one chain",
                 "frac": ach / peak, "traffic": TRAFFIC_TRAJ_PER_FRAME * per_step_frames,
-                "peak_source": f"{RK4_CHAIN_CYCLES} cycles of dependent instructions per step at {mhz:.0f} MHz",
+                "peak_source": f"estimate: {RK4_CHAIN_CYCLES} cycles of dependent instructions per step at {mhz:.0f} MHz",
+                "steps_per_s_of_binary64_pipe_measured": fp64_peak * 1e12 / (sms * 4) / (32 * RK4_FP64_INSTR),
+                "vs_binary64_pipe_measured": ach / (fp64_peak * 1e12 / (sms * 4) / (32 * RK4_FP64_INSTR)),
                 "per_launch_units": f"{per_step_frames} frames x one trajectory of {steps} RK4 steps + the D/B emission",
                 "timing": "one launch (trajectory + emission) with nothing else running",
                 "ms_per_launch_alone": ms, "ms_per_launch_in_timed_run": kern[k]["avg_launch_ms"],
