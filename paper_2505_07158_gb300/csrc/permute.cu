@@ -32,8 +32,8 @@ namespace {
 
 // CTA shapes.  Column pass: 512 threads at two CTAs per SM (the default; 1024 where the strip leaves room for one
 // CTA) or 256 at four; row pass: 256 threads held to six CTAs per SM (40 registers) or 128 at twelve.  The autotuner picks per frame shape
-// (fhd_set_cta_threads); on the 30-frame 1080p clip the defaults measured 0.269 / 0.259 ms per encrypt /
-// decrypt permutation call, 256-thread column-pass CTAs 0.326 / 0.368.
+// (fhd_set_cta_threads): a frame of a 30-frame 1080p clip both ways 16.2 us with the defaults at P = 16, 15.9 with 128-thread
+// row-pass CTAs, 22.6 with 256-thread column-pass CTAs; of a 4K batch, P = 32, 69.5, 68.0, 90.8, and 73.3 us with 512 threads.
 constexpr size_t kSmemPerSm = 233472, kSmemReserved = 1024;   // shared memory of an SM, and what each CTA adds
 constexpr int kStripThreads = 512;
 constexpr int kRowThreads = 256;
