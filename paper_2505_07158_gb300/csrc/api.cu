@@ -189,12 +189,12 @@ cudaError_t frame_alloc(uint8_t **p, size_t bytes, cudaStream_t s) {
     static bool tried[64] = {};
     int dev = 0;
     cudaMemPool_t pool = nullptr, def = nullptr;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    if (!capturing(s) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {   // under capture the graph allocates
         std::lock_guard<std::mutex> lk(mu);
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // another thread's stream may be under capture
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (!tried[dev]) {
             tried[dev] = true;
-            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // another stream may be under capture
-            cudaThreadExchangeStreamCaptureMode(&mode);
             cudaMemPoolProps props = {};
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
@@ -203,8 +203,6 @@ cudaError_t frame_alloc(uint8_t **p, size_t bytes, cudaStream_t s) {
             if (cudaMemPoolCreate(&pools[dev], &props) != cudaSuccess ||
                 cudaMemPoolSetAttribute(pools[dev], cudaMemPoolReuseAllowOpportunistic, &off) != cudaSuccess)
                 pools[dev] = nullptr;
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            cudaGetLastError();
         }
         pool = pools[dev];
         uint64_t want = 0, have = 0;
@@ -212,9 +210,10 @@ cudaError_t frame_alloc(uint8_t **p, size_t bytes, cudaStream_t s) {
             cudaMemPoolGetAttribute(def, cudaMemPoolAttrReleaseThreshold, &want) == cudaSuccess &&
             cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &have) == cudaSuccess && want != have)
             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &want);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (pool && cudaMallocFromPoolAsync((void **)p, bytes, pool, s) == cudaSuccess) return cudaSuccess;
+        cudaGetLastError();
     }
-    if (pool && cudaMallocFromPoolAsync((void **)p, bytes, pool, s) == cudaSuccess) return cudaSuccess;
-    cudaGetLastError();
     return cudaMallocAsync((void **)p, bytes, s);
 }
 

@@ -211,3 +211,52 @@ def test_decrypting_passes_on_many_streams():
     assert r.returncode == 0, r.stderr
     t = [float(x) for x in r.stdout.split("times")[1].split()]
     assert t[1] < 1.1 * t[0], t
+
+
+UNDER_CAPTURE = """
+import sys, threading, torch
+import paper_2505_07158_gb300 as fhd
+h, w, c = 61, 67, 3
+g = torch.Generator(device="cuda").manual_seed(1)
+F, B = (torch.randint(0, 256, (h, w, c), dtype=torch.uint8, device="cuda", generator=g) for _ in range(2))
+D = torch.randint(-32768, 32768, (c * (h + w),), dtype=torch.int16, device="cuda", generator=g)
+E, P, E2, P2 = (torch.zeros_like(F) for _ in range(4))
+s2 = torch.cuda.Stream()
+
+def both(e, p, s):
+    fhd.fhd_permute_encrypt(F, D, B, out=e, stream=s)
+    fhd.fhd_permute_decrypt(e, D, B, out=p, stream=s)
+
+x = torch.zeros(4, device="cuda")
+x += 1
+torch.cuda.synchronize()
+G = torch.cuda.CUDAGraph()
+with torch.cuda.graph(G, capture_error_mode="thread_local"):
+    if sys.argv[1] == "captured":
+        both(E, P, torch.cuda.current_stream())
+    else:   # another thread's first calls while this one captures
+        t = threading.Thread(target=both, args=(E2, P2, s2))
+        t.start()
+        t.join()
+        x += 1
+if sys.argv[1] == "captured":
+    for _ in range(2):
+        E.zero_(), P.zero_()
+        G.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(P, F)
+else:
+    torch.cuda.synchronize()
+    assert torch.equal(P2, F)
+both(E2, P2, s2)
+torch.cuda.synchronize()
+assert torch.equal(P2, F) and (sys.argv[1] != "captured" or torch.equal(E2, E))
+"""
+
+
+@pytest.mark.parametrize("who", ["captured", "beside"])
+def test_permutation_under_capture(who):
+    """A process's first calls captured into a graph, and its first calls beside another thread's capture."""
+    r = subprocess.run([sys.executable, "-c", UNDER_CAPTURE, who], capture_output=True, text=True, timeout=300,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0, r.stderr
