@@ -14,6 +14,8 @@ import paper_2505_07158_gb300 as fhd
 from paper_2505_07158_gb300 import _lib
 
 pytestmark = pytest.mark.gpu
+# the checked build's kernels take other times
+timed = pytest.mark.skipif(fhd.checked_requested(), reason="times of the default build")
 
 
 def fastest(fn, reps=6):
@@ -45,6 +47,7 @@ def noise(*shape, seed=1):
     return torch.randint(0, 256, shape, dtype=torch.uint8, device="cuda", generator=g)
 
 
+@timed
 def test_calls_on_more_streams_than_hardware_queues():
     """Twelve encryption calls of 8 frames on twelve streams (8 hardware queues by default): two rounds of the queues at
     most (1.9 times one round of 8 calls; 3.1 where a kernel held its queue)."""
@@ -83,6 +86,7 @@ def test_digests_of_pipelines_that_come_to_share_an_sm(nbytes):
             assert got.tobytes() == acc.to_bytes(32, "big")
 
 
+@timed
 def test_digest_time_of_pipelines_that_share_an_sm():
     """240 pipelines of two calls on 152 SMs against the 120 of one call, two lanes per message (1.2 times; 1.55
     where every pipeline keeps two lanes per message)."""
@@ -98,6 +102,7 @@ def pairs_of(count, h, w, npairs):
                         torch.randint(0, w - 1, (count, 3, npairs), device="cuda", generator=g)], dim=-1).int()
 
 
+@timed
 def test_correlation_time_of_many_frames():
     """1,025 pairs of each of 1,000 frames against 1,024: the pairs of a direction are not spread over more CTAs where the
     frames fill the GPU by themselves (equal; 5 times where they were)."""
@@ -122,6 +127,7 @@ def test_correlation_sums_by_any_number_of_ctas(count, npairs):
         assert torch.equal(sums[:, :, d], ref)
 
 
+@timed
 def test_local_entropy_time_of_flat_blocks():
     """100 blocks of 16 x 16 of each of 300 flat frames against noise frames: a flat block has one logarithm to take, a
     noise block a dozen (no dearer; 1.75 times where every count up to the largest
@@ -133,6 +139,7 @@ def test_local_entropy_time_of_flat_blocks():
     assert t[1] < 1.4 * t[0], t
 
 
+@timed
 def test_chain_time_at_gammas_beyond_the_attractors():
     """2,048 steps of LHCS_m at a gamma whose states leave the integer step's ranges, against one that it does not take
     at all, binary64 throughout (equal; 1.8 times where every step was tried on the integer pipes first)."""
@@ -144,6 +151,7 @@ def test_chain_time_at_gammas_beyond_the_attractors():
     assert t[1] < 1.25 * t[0], t
 
 
+@timed
 def test_worker_pair_time_of_short_slices():
     """304 pairs of 21 steps each from iterates off the attractor against 305 x 2, which the binary64 kernel takes: as
     long (1.06 times; 1.28 where the short slices took the integer step)."""
@@ -167,6 +175,7 @@ def test_worker_pairs_on_both_sides_of_the_short_slices(n, w):
     assert np.array_equal(B.cpu().numpy().reshape(-1), np.asarray(B_ref).reshape(-1))
 
 
+@timed
 def test_chain_time_on_the_attractor():
     """The integer step is what runs, and few of its steps are done again: 2,048 steps at gamma = -0.9123 against -1, which
     it does not take (0.68 times)."""
@@ -201,6 +210,7 @@ print("times", *t)
 """
 
 
+@timed
 def test_decrypting_passes_on_many_streams():
     """64 decrypting passes on 32 streams with hardware queues of their own against the same 64 on one stream: half the
     time (1.8 times it where the temporary frames came from CUDA's default pool, whose search for other streams' freed
